@@ -37,96 +37,122 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
          (static_cast<uint32_t>(__bfloat16_as_ushort(b)) << 16);
 }
 
-// Upstream top-k weight gradient of one token, folded into per-expert terms:
-//   dt[e] = sum over top-k slots i with idx_i == e of dtil_i, and gdt = sum_i g_{idx_i} dtil_i,
-// where dtil_i = d_i (raw weights) or (d_i - sum_i' d_i' w_i') / G (renormalised, G = sum g_sel).
-struct Upstream {
-  int idx[kMaxTopK];
-  float dtil[kMaxTopK];
-  float gdt;
+// One token's top-k slots, spread over the GS-lane thread group that holds the token: lane c keeps
+// slots c, c + GS, ... (expert -1: no slot) with the upstream gradients of their weights (kUp).
+// Loaded with the token's other inputs and handed round by shuffles; every lane holding all slots
+// and gathering their gate values from memory took 15 of the 22 us of the preparation kernel on
+// 32768 tokens (E = 64, k = 6).
+template <int GS>
+struct TopkSlots {
+  static constexpr int kPer = (kMaxTopK + GS - 1) / GS;
+  int idx[kPer];
+  float d[kPer];
 };
 
-__device__ __forceinline__ void load_upstream(const BwdParams& p, int j, Upstream& u) {
+template <int GS, bool kUp>
+__device__ __forceinline__ void load_slots(const BwdParams& p, int j, bool valid, int c, TopkSlots<GS>& u) {
   const int k = p.dm.k;
-  float gsel[kMaxTopK], d[kMaxTopK];
-  float G = 0.f, dw = 0.f;
-  const float* g = p.ws.gsave + static_cast<size_t>(j) * p.dm.E;
-  const float ginv = p.ws.ginv[j];
 #pragma unroll
-  for (int i = 0; i < kMaxTopK; ++i) {
-    u.idx[i] = -1;
-    u.dtil[i] = 0.f;
-    gsel[i] = 0.f;
-    d[i] = 0.f;
-    if (i < k) {
-      u.idx[i] = p.topk_idx[static_cast<size_t>(j) * k + i];
-      d[i] = p.d_topk_w[static_cast<size_t>(j) * k + i];
-      const int e = u.idx[i];
-      gsel[i] = (e >= 0 && e < p.dm.E) ? g[e] * ginv : 0.f;
-      G += gsel[i];
-    }
+  for (int i = 0; i < TopkSlots<GS>::kPer; ++i) {
+    const int s = i * GS + c;
+    const bool in = valid && s < k;
+    u.idx[i] = in ? __ldg(p.topk_idx + static_cast<size_t>(j) * k + s) : -1;
+    u.d[i] = kUp && in ? __ldg(p.d_topk_w + static_cast<size_t>(j) * k + s) : 0.f;
   }
-  if (p.dm.renorm) {
-#pragma unroll
-    for (int i = 0; i < kMaxTopK; ++i)
-      if (i < k) dw += d[i] * gsel[i] / G;
-  }
-  float gdt = 0.f;
-#pragma unroll
-  for (int i = 0; i < kMaxTopK; ++i) {
-    if (i < k) {
-      u.dtil[i] = p.dm.renorm ? (d[i] - dw) / G : d[i];
-      gdt += gsel[i] * u.dtil[i];
-    }
-  }
-  u.gdt = gdt;
 }
 
-__device__ __forceinline__ float upstream_at(const Upstream& u, int k, int e) {
-  float r = 0.f;
+// Adds that gradient at the thread's N experts (eidx; negative: none) to dz. With a_e = sum of the
+// slots' gradients d_i with idx_i == e and n_e their number, the derivative at the gate value is
+//   t_e = a_e (raw weights) or (a_e - n_e sum_e' g_e' a_e' / G) / G (renormalised, G = sum n_e g_e),
+// then through the gate: g_e (t_e - sum_e' g_e' t_e') for the softmax, fac_e g_e t_e for the
+// sigmoid. The sums over experts are shuffles inside the GS-lane group.
+template <int GS, int N>
+__device__ __forceinline__ void add_upstream(const BwdParams& p, const TopkSlots<GS>& u, const int (&eidx)[N],
+                                             const float (&g)[N], const float (&fac)[N], bool gate, float (&dz)[N]) {
+  const int k = p.dm.k;
+  float a[N], n[N];
 #pragma unroll
-  for (int i = 0; i < kMaxTopK; ++i)
-    if (i < k && u.idx[i] == e) r += u.dtil[i];
-  return r;
+  for (int i = 0; i < N; ++i) a[i] = n[i] = 0.f;
+#pragma unroll
+  for (int q = 0; q < TopkSlots<GS>::kPer; ++q) {
+#pragma unroll
+    for (int r = 0; r < GS; ++r) {
+      if (q * GS + r >= k) break;                     // the same for every thread
+      const int e = __shfl_sync(0xffffffffu, u.idx[q], r, GS);
+      const float d = __shfl_sync(0xffffffffu, u.d[q], r, GS);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const bool hit = e >= 0 && e == eidx[i];
+        a[i] += hit ? d : 0.f;
+        n[i] += hit ? 1.f : 0.f;
+      }
+    }
+  }
+  float G = 0.f, ga = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    G = fmaf(n[i], g[i], G);
+    ga = fmaf(g[i], a[i], ga);
+  }
+#pragma unroll
+  for (int o = 1; o < GS; o <<= 1) {
+    G += __shfl_xor_sync(0xffffffffu, G, o);
+    ga += __shfl_xor_sync(0xffffffffu, ga, o);
+  }
+  if (p.dm.renorm) {
+    const float iG = G > 0.f ? 1.f / G : 0.f, dw = ga * iG;
+    ga = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      a[i] = fmaf(-n[i], dw, a[i]) * iG;
+      ga = fmaf(g[i], a[i], ga);
+    }
+#pragma unroll
+    for (int o = 1; o < GS; o <<= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i) dz[i] = gate ? fmaf(fac[i] * g[i], a[i], dz[i]) : fmaf(g[i], a[i] - ga, dz[i]);
 }
 
 // Gradient of the bin-level balance loss (eq. 16) at one token's logits, added to dz[N] of the
 // thread's N experts (g: their gate values, be: their bins (-1: none), fe: their f_e, fac: the
 // gate's own factor, 1 for the softmax and 1 - s for the sigmoid): for every bin k the token
-// routes to, dz_e += a_k h_e (f_e - sum_{e' in B_k} f_e' h_e') fac_e with h = g / (bin sum). The bin sums run over the token's GS-lane thread group (xor shuffles); every lane takes
-// the same k iterations, and a bin repeated among the token's selections adds nothing again.
+// routes to, dz_e += a_k h_e (f_e - sum_{e' in B_k} f_e' h_e') fac_e with h = g / (bin sum). The
+// bin sums run over the token's GS-lane thread group (xor shuffles); every lane takes the same k
+// iterations, and a bin repeated among the token's selections adds nothing again.
 template <int GS, int N>
-__device__ __forceinline__ void add_balance_grad(const BwdParams& p, int j, bool valid, const float (&g)[N],
+__device__ __forceinline__ void add_balance_grad(const BwdParams& p, const TopkSlots<GS>& slots, const float (&g)[N],
                                                  const int (&be)[N], const float (&fe)[N],
                                                  const float (&fac)[N], float (&dz)[N]) {
   const int k = p.dm.k;
-  int seen[kMaxTopK];
+  uint32_t seen = 0u;
 #pragma unroll
-  for (int s = 0; s < kMaxTopK; ++s) {
-    if (s >= k) break;
-    const int es = valid ? __ldg(p.topk_idx + static_cast<size_t>(j) * k + s) : -1;
-    const int bs = (es >= 0 && es < p.dm.E) ? (p.dm.contig_bins ? es / p.dm.N_B : __ldg(p.ws.expert_bin + es)) : -1;
-    seen[s] = bs;
-    bool dup = bs < 0;
+  for (int q = 0; q < TopkSlots<GS>::kPer; ++q) {
+    const int es = slots.idx[q];                      // bins of this lane's own slots
+    const int own = (es >= 0 && es < p.dm.E) ? __ldg(p.ws.expert_bin + es) : -1;
 #pragma unroll
-    for (int s2 = 0; s2 < kMaxTopK; ++s2)
-      if (s2 < s) dup = dup || seen[s2] == bs;
-    float v = 0.f, w = 0.f;
+    for (int r = 0; r < GS; ++r) {
+      if (q * GS + r >= k) break;                     // the same for every thread
+      const int bs = __shfl_sync(0xffffffffu, own, r, GS);
+      const bool dup = bs < 0 || ((seen >> (bs & 31)) & 1u);
+      if (bs >= 0) seen |= 1u << bs;
+      float v = 0.f, w = 0.f;
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-      v += be[i] == bs ? g[i] : 0.f;
-      w += be[i] == bs ? fe[i] * g[i] : 0.f;
-    }
+      for (int i = 0; i < N; ++i) {
+        v += be[i] == bs ? g[i] : 0.f;
+        w += be[i] == bs ? fe[i] * g[i] : 0.f;
+      }
 #pragma unroll
-    for (int o = 1; o < GS; o <<= 1) {
-      v += __shfl_xor_sync(0xffffffffu, v, o);
-      w += __shfl_xor_sync(0xffffffffu, w, o);
-    }
-    if (!dup && v > 0.f) {
-      const float a = __ldg(p.ws.bal_a + bs), iv = 1.f / v, phi = w * iv;
+      for (int o = 1; o < GS; o <<= 1) {
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+        w += __shfl_xor_sync(0xffffffffu, w, o);
+      }
+      if (!dup && v > 0.f) {
+        const float a = __ldg(p.ws.bal_a + bs), iv = 1.f / v, phi = w * iv;
 #pragma unroll
-      for (int i = 0; i < N; ++i)
-        if (be[i] == bs) dz[i] = fmaf(a * g[i] * iv * fac[i], fe[i] - phi, dz[i]);
+        for (int i = 0; i < N; ++i)
+          if (be[i] == bs) dz[i] = fmaf(a * g[i] * iv * fac[i], fe[i] - phi, dz[i]);
+      }
     }
   }
 }
@@ -193,7 +219,7 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
   pdl_wait();                                         // scores and tables of the forward
   pdl_trigger();
   const Dims& dm = p.dm;
-  const int E = dm.E, K = dm.K, k = dm.k;
+  const int E = dm.E, K = dm.K;
   constexpr int kEp = TPT * 8;
   constexpr int kGroups = 256 / TPT;                  // token groups per block and set
   const int c = threadIdx.x % TPT;
@@ -211,6 +237,11 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
   float ginv[kDzRep];
   float2 m[kDzRep];
   int smp[kDzRep];
+  TopkSlots<TPT> slots[kDzRep];
+  // consecutive bins: the thread's experts lie in bin b0 up to expert e0 + nb0 and in bin b1 after
+  // (one division per thread: a division per expert made this kernel issue-bound)
+  const int b0 = dm.contig_bins ? e0 / dm.N_B : 0, nb0 = (b0 + 1) * dm.N_B - e0;
+  const int b1 = nb0 < 8 ? b0 + 1 : b0;
   const bool vec = (E & 3) == 0 && e0 + 8 <= E;
   // the balance term (eq. 16) when smoes_bin_balance armed this backward
   const bool bal = kBal && p.topk_idx != nullptr && __ldcg(p.ws.bal_flag) != 0u;
@@ -222,7 +253,7 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
     be[i] = -1;
     fe[i] = 0.f;
     if (bal && e < E) {
-      be[i] = dm.contig_bins ? e / dm.N_B : __ldg(p.ws.expert_bin + e);
+      be[i] = dm.contig_bins ? (i < nb0 ? b0 : b1) : __ldg(p.ws.expert_bin + e);
       fe[i] = __ldg(p.ws.bal_f + e);
     }
   }
@@ -248,6 +279,7 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
       m[q] = __ldg(reinterpret_cast<const float2*>(p.M) + j[q]);
       smp[q] = __ldg(p.ws.token_sample + j[q]);
     }
+    if (kUp || bal) load_slots<TPT, kUp>(p, j[q], valid[q], c, slots[q]);
   }
 #pragma unroll
   for (int q = 0; q < kDzRep; ++q) {
@@ -261,11 +293,10 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
       // the sample's coefficient table was written by the forward kernel and is read-only here
       const float* tb = p.ws.tabs + static_cast<size_t>(smp[q]) * 3 * K;
       if (dm.contig_bins && e0 + 8 <= E) {
-        const int b0 = e0 / dm.N_B, b1 = (e0 + 7) / dm.N_B;
         const float u0 = __ldg(tb + 2 * K + b0) + dv * __ldg(tb + b0) + dt * __ldg(tb + K + b0);
         const float u1 = __ldg(tb + 2 * K + b1) + dv * __ldg(tb + b1) + dt * __ldg(tb + K + b1);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) u[i] = (e0 + i) / dm.N_B == b0 ? u0 : u1;
+        for (int i = 0; i < 8; ++i) u[i] = i < nb0 ? u0 : u1;
       } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -281,16 +312,8 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
     for (int i = 0; i < 8; ++i) eidx[i] = e0 + i < E ? e0 + i : -2;
     float dz[8], fac[8];
     mi_grad<TPT, 8, kVar>(p, j[q], valid[q], eidx, raw, g, u, fac, dz);
-    if (kUp && valid[q]) {
-      Upstream up;
-      load_upstream(p, j[q], up);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (e0 + i < E)
-          dz[i] += (kVar && dm.gate) ? fac[i] * g[i] * upstream_at(up, k, e0 + i)   // diagonal
-                                     : g[i] * (upstream_at(up, k, e0 + i) - up.gdt);
-    }
-    if (kBal && bal) add_balance_grad<TPT, 8>(p, j[q], valid[q], g, be, fe, fac, dz);
+    if (kUp) add_upstream<TPT, 8>(p, slots[q], eidx, g, fac, kVar && dm.gate, dz);
+    if (kBal && bal) add_balance_grad<TPT, 8>(p, slots[q], g, be, fe, fac, dz);
     if (valid[q] && p.dlogits) {
       float* dl = p.dlogits + static_cast<size_t>(j[q]) * E;
       if (vec) {
@@ -616,7 +639,7 @@ k_router_bwd_f32(const BwdParams p) {
   pdl_wait();
   pdl_trigger();
   const Dims& dm = p.dm;
-  const int E = dm.E, K = dm.K, k = dm.k;
+  const int E = dm.E, K = dm.K;
   const int nck = (dm.d + kF32Cols - 1) / kF32Cols;
   const int tile = blockIdx.x / nck, ck = blockIdx.x % nck;
   constexpr int kZs = EB + 4;                        // dz row stride (16-byte aligned rows)
@@ -635,9 +658,11 @@ k_router_bwd_f32(const BwdParams p) {
       dt = p.M[2 * static_cast<size_t>(j) + 1] - 0.5f;
       tb = p.ws.tabs + static_cast<size_t>(s) * 3 * K;
     }
-    Upstream up;
-    const bool has_up = valid && p.d_topk_w != nullptr;
-    if (has_up) load_upstream(p, j, up);
+    TopkSlots<4> slots;
+    const bool has_up = p.d_topk_w != nullptr;
+    const bool bal = p.topk_idx && __ldcg(p.ws.bal_flag) != 0u;   // the balance term (eq. 16); block-uniform
+    if (has_up) load_slots<4, true>(p, j, valid, qd, slots);
+    else if (bal) load_slots<4, false>(p, j, valid, qd, slots);
     const float* g = p.ws.gsave + static_cast<size_t>(valid ? j : 0) * E;
     const float ginv = valid ? p.ws.ginv[j] : 0.f;
     // the token's 4-thread group holds experts qd, qd + 4, ...
@@ -655,17 +680,11 @@ k_router_bwd_f32(const BwdParams p) {
       uq[i] = in ? tb[2 * K + bq[i]] + dv * tb[bq[i]] + dt * tb[K + bq[i]] : 0.f;
     }
     mi_grad<4, NQ>(p, j, valid, eidx, raw, gq, uq, fac, dzv);
-    if (has_up) {
-#pragma unroll
-      for (int i = 0; i < NQ; ++i)
-        if (eidx[i] >= 0)
-          dzv[i] += dm.gate ? fac[i] * gq[i] * upstream_at(up, k, eidx[i])
-                            : gq[i] * (upstream_at(up, k, eidx[i]) - up.gdt);
-    }
-    if (p.topk_idx && __ldcg(p.ws.bal_flag) != 0u) {   // the balance term (eq. 16); block-uniform
+    if (has_up) add_upstream<4, NQ>(p, slots, eidx, gq, fac, dm.gate != 0, dzv);
+    if (bal) {
 #pragma unroll
       for (int i = 0; i < NQ; ++i) fq[i] = bq[i] >= 0 ? p.ws.bal_f[eidx[i]] : 0.f;
-      add_balance_grad<4, NQ>(p, j, valid, gq, bq, fq, fac, dzv);
+      add_balance_grad<4, NQ>(p, slots, gq, bq, fq, fac, dzv);
     }
 #pragma unroll
     for (int i = 0; i < EB / 4; ++i) {
