@@ -12,6 +12,7 @@
 namespace smoes {
 int perm_blocks(int T, int k);
 int perm_rounds(int T, int k);
+int stats_blocks(int T, int n_sms);
 }
 
 using namespace smoes;
@@ -44,6 +45,7 @@ struct smoes_plan_s {
   int perm_nblocks = 0;
   int dcoef = 256;       // Gaussian coefficient vectors padded to 256 features
   int stat_blocks = 1;   // blocks of the statistics pass (one partial each)
+  int bal_blocks = 1;    // blocks of the balance pass (one partial each)
   bool contig_bins = false;
   uint64_t limit_ns = kWaitLimitNs;   // bounded device waits
   bool balance_armed = false;         // smoes_bin_balance enqueued since the last forward
@@ -380,16 +382,17 @@ smoes_status smoes_plan_create(const smoes_router_desc* desc, smoes_plan* out) {
   L.fperm = take(sizeof(int32_t) * static_cast<size_t>(std::max(P->n_sms, 1)) * K);   // per-CTA counts
   L.attn_part = take(sizeof(float) * static_cast<size_t>(T) * std::max(0, d.attn_max_heads));
   L.gcoef = take(sizeof(float) * (2 * static_cast<size_t>(P->dcoef) + P->dcoef / 256));
-  P->stat_blocks = std::max(1, std::min(2 * P->n_sms, (T + 63) / 64));
+  P->stat_blocks = stats_blocks(T, P->n_sms);
+  P->bal_blocks = std::max(1, std::min(2 * P->n_sms, (T + 63) / 64));
   L.stat_part = take(sizeof(float) * 4 * static_cast<size_t>(P->stat_blocks) * d.d);
   L.stat_nvis = take(sizeof(int32_t) * static_cast<size_t>(P->stat_blocks));
   L.stat_n0 = take(sizeof(double) * 2);
   L.gmmcoef = take(sizeof(float) * kGmmMaxForms * (2 * static_cast<size_t>(P->dcoef) + P->dcoef / 256));
   L.bal_f = take(sizeof(float) * E);
   L.bal_a = take(sizeof(float) * K);
-  L.bal_h = take(sizeof(float) * static_cast<size_t>(P->stat_blocks) * E);
-  L.bal_s = take(sizeof(int32_t) * static_cast<size_t>(P->stat_blocks) * E);
-  L.bal_u = take(sizeof(int32_t) * static_cast<size_t>(P->stat_blocks) * K);
+  L.bal_h = take(sizeof(float) * static_cast<size_t>(P->bal_blocks) * E);
+  L.bal_s = take(sizeof(int32_t) * static_cast<size_t>(P->bal_blocks) * E);
+  L.bal_u = take(sizeof(int32_t) * static_cast<size_t>(P->bal_blocks) * K);
   L.f32_part = take(d.dtype == SMOES_F32 ? sizeof(float) * static_cast<size_t>(P->n_groups) *
                                                f32_chunks(d.d) * (E + 1) * 128 : 0);
   L.total = o;
@@ -779,6 +782,8 @@ smoes_status smoes_gaussian_stats_update(smoes_plan P, const void* X, const uint
   p.part = reinterpret_cast<float*>(b + P->L.stat_part);
   p.nvis = reinterpret_cast<int32_t*>(b + P->L.stat_nvis);
   p.N0 = reinterpret_cast<double*>(b + P->L.stat_n0);
+  p.status = reinterpret_cast<uint32_t*>(b + P->L.status);
+  p.limit_ns = P->limit_ns;
   return cuda_status(launch_stats_update(p, d.dtype == SMOES_BF16, stream));
 }
 
@@ -801,7 +806,7 @@ smoes_status smoes_bin_balance(smoes_plan P, const int32_t* topk_idx, float loss
   p.k = d.k;
   p.K = d.n_bins;
   p.N_B = P->N_B;
-  p.G = P->stat_blocks;
+  p.G = P->bal_blocks;
   p.gsave = v.gsave;
   p.topk_idx = topk_idx;
   p.expert_bin = v.expert_bin;

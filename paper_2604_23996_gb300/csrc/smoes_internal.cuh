@@ -210,6 +210,8 @@ struct StatsParams {
   float* part;
   int32_t* nvis;
   double* N0;                // [2] copy of N_{t-1}
+  uint32_t* status;
+  uint64_t limit_ns;
 };
 
 // Bin-level load-balance loss (eq. 16) from the forward's saved scores: per-block partials

@@ -75,6 +75,30 @@ def test_gaussian_stats_update_several_steps(bd, d, dtype, beta):
         print(f"d={d} step {seed}: rel err S_mu {e_mu:.2e} S_var {e_var:.2e}")
 
 
+@pytest.mark.parametrize("T,d,dtype", [(1, 8, torch.bfloat16), (33, 264, torch.bfloat16), (5000, 4104, torch.bfloat16),
+                                       (20000, 16, torch.float32), (700, 2056, torch.float32), (400, 512, torch.float32)])
+def test_stats_splits_of_rows_and_features(bd, T, d, dtype):
+    # one row, row groups of one warp and of eight, stages that end in a ragged chunk, several
+    # feature passes; a carried state whose vision count is subnormal (its reciprocal overflows)
+    dev = "cuda"
+    X, is_vis = _batch(T + d, T, d, dtype, 0.4)
+    rng = np.random.default_rng(d)
+    N = np.array([1e-310, 700.0])
+    S_mu, S_var = N[:, None] * rng.standard_normal((2, d)), N[:, None] * rng.uniform(0.5, 2.0, (2, d))
+    Nt, Sm, Sv = (torch.from_numpy(a.copy()).to(dev) for a in (N, S_mu, S_var))
+    r = _plan(bd, T, d, dtype)
+    assert bd.smoes_gaussian_stats_update(r.plan, X.to(dev), torch.from_numpy(is_vis).to(dev), 0.9, Nt, Sm, Sv,
+                                          None, None, r.ws) == 0
+    assert r.device_status()[0] == 0
+    ref = O.gaussian_stats_update((N, S_mu, S_var), X.double().numpy(), is_vis, 0.9)
+    np.testing.assert_allclose(Nt.cpu().numpy(), ref[0], rtol=1e-12, atol=0)
+    for m in range(2):                          # per modality: an absent one decays to ~1e-310
+        if is_vis.sum() == (0 if m == 0 else T):
+            continue
+        assert_tensor_close(Sm[m].cpu().numpy(), ref[1][m], f"S_mu[{m}]")
+        assert_tensor_close(Sv[m].cpu().numpy(), ref[2][m], f"S_var[{m}]")
+
+
 def test_first_update_gives_the_batch_moments(bd):
     # from the empty state one update leaves mu = batch mean and var = biased batch variance per
     # hard modality (the statistics the timed workloads feed the score)
