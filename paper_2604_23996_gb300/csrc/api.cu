@@ -593,18 +593,18 @@ smoes_status smoes_attention_fwd(smoes_plan P, const smoes_attn_args* args, cons
   p.x_norm = a.x_norm;
   p.M = M;
   p.part = v.attn_part;
-  p.ticket = v.attn_ticket;
   p.status = v.status;
   p.n_qtiles = a.S / 128;
   p.n_items = a.B * a.H * p.n_qtiles;
   p.limit_ns = P->limit_ns;
   fp.Hkv = n_kv_heads;
-  CUtensorMap tq, tk, tv, to;
+  fp.O = O;
+  CUtensorMap tq, tk, tv;
   const uint64_t rq = static_cast<uint64_t>(a.B) * a.H * a.S, rk = static_cast<uint64_t>(a.B) * n_kv_heads * a.S;
   if (!encode_bf16_2d(&tq, a.Q, rq, a.hd, 128, 64, true) || !encode_bf16_2d(&tk, a.K, rk, a.hd, 128, 64, true) ||
-      !encode_bf16_2d(&tv, V, rk, a.hd, 128, 64, true) || !encode_bf16_2d(&to, O, rq, a.hd, 128, 64, true))
+      !encode_bf16_2d(&tv, V, rk, a.hd, 128, 64, true))
     return SMOES_ERR_CUDA;
-  const cudaError_t e = launch_attn_fwd(fp, tq, tk, tv, to, P->n_sms, stream);
+  const cudaError_t e = launch_attn_fwd(fp, tq, tk, tv, P->n_sms, stream);
   if (e == cudaErrorNotSupported) return SMOES_ERR_UNSUPPORTED;
   return cuda_status(e);
 }

@@ -118,3 +118,28 @@ def test_attention_forward_limits(bd):
                 is_vision=torch.from_numpy(aw.is_vision).cuda())
     assert bd.smoes_attention_fwd(r.plan, attn, V.cuda(), 3, Ot, M, r.ws) == -1     # H % H_kv != 0
     assert bd.smoes_attention_fwd(r.plan, dict(attn, hd=64), V.cuda(), 4, Ot, M, r.ws) == -2
+
+
+@pytest.mark.parametrize("B,H,Hkv,S,case", [(1, 2, 1, 640, "rising"), (3, 8, 8, 128, "padded"), (20, 16, 16, 256, "runs"),
+                                            (1, 4, 4, 384, "scattered"), (1, 2, 2, 256, "negative")])
+def test_forward_key_chunks_and_rescale(bd, B, H, Hkv, S, case):
+    # an odd number of query tiles (a pair of one), many short items per CTA, keys whose bias and score
+    # change inside a 32-key chunk or are -inf, logits that grow by far more than 2^8 along the keys
+    # (the running maximum is raised, O rescaled), and a logit scale whose maximum is not the products'
+    aw, K, V = _case(B, H, Hkv, S, seed=900 + S + H, n_image=S // 4)
+    rng = np.random.default_rng(S)
+    if case == "rising":
+        aw.key_bias = np.tile(np.linspace(0.0, 60.0, S, dtype=np.float32), B)
+    elif case == "padded":                                # every query keeps key 0
+        aw.key_bias = np.where(np.arange(B * S) % S > 90, -np.inf, 0.0).astype(np.float32)
+    elif case == "scattered":
+        aw.is_vision = (rng.random(B * S) < 0.5).astype(np.uint8)
+        aw.key_bias = rng.standard_normal(B * S).astype(np.float32)
+    elif case == "negative":
+        aw.sm_scale = -aw.sm_scale
+    _, _, Og, Mg = _run(bd, aw, K, V, Hkv)
+    Oref, mass = O.attention_forward_with_mass(aw.Q.double().numpy(), K.double().numpy(), V.double().numpy(),
+                                               aw.is_vision.reshape(B, S).astype(np.float64), aw.sm_scale, True,
+                                               aw.key_bias.reshape(B, S))
+    _check_O(Og, Oref, float(V.float().abs().max()), "O")
+    assert_tensor_close(Mg[:, 0], mass.reshape(-1), "vision mass")
