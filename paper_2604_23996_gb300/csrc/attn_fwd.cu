@@ -395,7 +395,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   float* mxs = reinterpret_cast<float*>(base + L.mx);
   float* mrg = reinterpret_cast<float*>(base + L.mrg);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int n_items = ((p.n_qtiles + 1) / 2) * p.B * p.H;
   WaitCtx wc{abort_flag, p.status, p.limit_ns};
   if (threadIdx.x == 0) {
@@ -436,7 +436,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
+    {
       const int G = p.H / fp.Hkv;         // query heads per key/value head
       int st = 0, vst = 0;
       uint32_t ph = 0, vph = 0;
@@ -449,27 +449,36 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         const AttnItem w = decode_item(p, item);
         const int row0 = (w.b * p.H + w.h) * p.S, krow0 = (w.b * fp.Hkv + w.h / G) * p.S;
         for (int t = 0; t < w.nq && ok; ++t) {
-          if (!wait_idle(q_empty + t, (static_cast<uint32_t>(nqt[t]) & 1u) ^ 1u, wc)) { ok = false; break; }
+          if (!warp_wait(q_empty + t, (static_cast<uint32_t>(nqt[t]) & 1u) ^ 1u, wc)) { ok = false; break; }
           ++nqt[t];
-          mbar_arrive_expect_tx(q_full + t, kAttnTileBytes);
-          uint8_t* qd = qs + t * kAttnTileBytes;
-          tma_load_2d(qd, &tmQ, q_full + t, 0, row0 + (w.qt0 + t) * kAttnTile);
-          tma_load_2d(qd + kAttnTileBytes / 2, &tmQ, q_full + t, 64, row0 + (w.qt0 + t) * kAttnTile);
+          if (elect_one()) {
+            mbar_arrive_expect_tx(q_full + t, kAttnTileBytes);
+            uint8_t* qd = qs + t * kAttnTileBytes;
+            tma_load_2d(qd, &tmQ, q_full + t, 0, row0 + (w.qt0 + t) * kAttnTile);
+            tma_load_2d(qd + kAttnTileBytes / 2, &tmQ, q_full + t, 64, row0 + (w.qt0 + t) * kAttnTile);
+          }
+          __syncwarp();
         }
         const int nkb = kblocks_of(p, w.qt0 + w.nq - 1);
         for (int kb = 0; kb < nkb && ok; ++kb) {
-          if (!wait_idle(k_empty + st, ph ^ 1u, wc)) { ok = false; break; }
-          uint8_t* kd = ks + st * kAttnTileBytes;
-          mbar_arrive_expect_tx(k_full + st, kAttnTileBytes);
-          tma_load_2d(kd, &tmK, k_full + st, 0, krow0 + kb * kAttnTile);
-          tma_load_2d(kd + kAttnTileBytes / 2, &tmK, k_full + st, 64, krow0 + kb * kAttnTile);
+          if (!warp_wait(k_empty + st, ph ^ 1u, wc)) { ok = false; break; }
+          if (elect_one()) {
+            uint8_t* kd = ks + st * kAttnTileBytes;
+            mbar_arrive_expect_tx(k_full + st, kAttnTileBytes);
+            tma_load_2d(kd, &tmK, k_full + st, 0, krow0 + kb * kAttnTile);
+            tma_load_2d(kd + kAttnTileBytes / 2, &tmK, k_full + st, 64, krow0 + kb * kAttnTile);
+          }
+          __syncwarp();
           ++nk;
           if (++st == kKStages) { st = 0; ph ^= 1u; }
-          if (!wait_idle(v_empty + vst, vph ^ 1u, wc)) { ok = false; break; }
-          uint8_t* vd = vs + vst * kAttnTileBytes;
-          mbar_arrive_expect_tx(v_full + vst, kAttnTileBytes);
-          tma_load_2d(vd, &tmV, v_full + vst, 0, krow0 + kb * kAttnTile);
-          tma_load_2d(vd + kAttnTileBytes / 2, &tmV, v_full + vst, 64, krow0 + kb * kAttnTile);
+          if (!warp_wait(v_empty + vst, vph ^ 1u, wc)) { ok = false; break; }
+          if (elect_one()) {
+            uint8_t* vd = vs + vst * kAttnTileBytes;
+            mbar_arrive_expect_tx(v_full + vst, kAttnTileBytes);
+            tma_load_2d(vd, &tmV, v_full + vst, 0, krow0 + kb * kAttnTile);
+            tma_load_2d(vd + kAttnTileBytes / 2, &tmV, v_full + vst, 64, krow0 + kb * kAttnTile);
+          }
+          __syncwarp();
           ++nv;
           if (++vst == kVStages) { vst = 0; vph ^= 1u; }
         }
@@ -486,7 +495,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
       const uint32_t id_s = idesc_bf16(kAttnTile, kAttnTile, false, false);   // S = Q K^T (both K-major)
       const uint32_t id_o = idesc_bf16(kAttnTile, kAttnHd, false, true);      // O += P V (V MN-major)
       int st = 0, vst = 0;
@@ -506,53 +515,61 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
         // over the weights it has read (the MMAs of one thread run in order); the other tile's
         // softmax runs meanwhile
         for (int j = 0; j <= nkb && ok; ++j) {
-          if (j < nkb && !mbar_wait(k_full + st, ph, wc)) { ok = false; break; }
-          if (j > 0 && !mbar_wait(v_full + vst, vph, wc)) { ok = false; break; }
+          if (j < nkb && !warp_wait(k_full + st, ph, wc)) { ok = false; break; }
+          if (j > 0 && !warp_wait(v_full + vst, vph, wc)) { ok = false; break; }
           for (int t = 0; t < w.nq && ok; ++t) {
             const uint32_t ts = tmem + static_cast<uint32_t>(t * kAttnTile);   // S, then P
             if (j > 0 && j <= nb[t]) {
               const uint32_t d = tmem + 256u + static_cast<uint32_t>(t * kAttnHd);
               const uint32_t vb = smem_u32(vs + vst * kAttnTileBytes);
               for (int hf = 0; hf < 2; ++hf) {
-                if (!mbar_wait(p_full + 2 * t + hf, static_cast<uint32_t>(blk[t] - 1) & 1u, wc)) { ok = false; break; }
-                if (j == 1 && hf == 0 && !mbar_wait(o_empty + t, (static_cast<uint32_t>(nqt[t] - 1) & 1u) ^ 1u, wc)) { ok = false; break; }
+                if (!warp_wait(p_full + 2 * t + hf, static_cast<uint32_t>(blk[t] - 1) & 1u, wc)) { ok = false; break; }
+                if (j == 1 && hf == 0 && !warp_wait(o_empty + t, (static_cast<uint32_t>(nqt[t] - 1) & 1u) ^ 1u, wc)) { ok = false; break; }
                 tc_fence_after();
+                if (elect_one()) {
 #pragma unroll
-                for (int k4 = 0; k4 < 4; ++k4) {             // K = 16 keys per step
-                  const int kk = 4 * hf + k4;
-                  umma_bf16_ta(d, ts + 8u * kk, sdesc_sw128(vb + kk * 2048, kAttnTileBytes / 2, 1024), id_o,
-                               (j > 1 || kk > 0) ? 1u : 0u);
+                  for (int k4 = 0; k4 < 4; ++k4) {           // K = 16 keys per step
+                    const int kk = 4 * hf + k4;
+                    umma_bf16_ta(d, ts + 8u * kk, sdesc_sw128(vb + kk * 2048, kAttnTileBytes / 2, 1024), id_o,
+                                 (j > 1 || kk > 0) ? 1u : 0u);
+                  }
+                  if (hf == 1 && j == nb[t]) umma_commit(o_full + t);
                 }
+                __syncwarp();
               }
               if (!ok) break;
-              if (j == nb[t]) umma_commit(o_full + t);
             }
             if (j < nb[t]) {
-              if (j == 0 && !mbar_wait(q_full + t, static_cast<uint32_t>(nqt[t]++) & 1u, wc)) { ok = false; break; }
+              if (j == 0 && !warp_wait(q_full + t, static_cast<uint32_t>(nqt[t]++) & 1u, wc)) { ok = false; break; }
               tc_fence_after();
               const uint32_t qa = smem_u32(qs + t * kAttnTileBytes), kb = smem_u32(ks + st * kAttnTileBytes);
+              if (elect_one()) {
 #pragma unroll
-              for (int kk = 0; kk < kAttnHd / 16; ++kk) {    // K = 16 of the head dimension per step
-                const uint32_t off = (kk >> 2) * (kAttnTileBytes / 2) + (kk & 3) * 32;
-                umma_bf16(ts, sdesc_sw128(qa + off, 16, 1024), sdesc_sw128(kb + off, 16, 1024), id_s, kk > 0 ? 1u : 0u);
+                for (int kk = 0; kk < kAttnHd / 16; ++kk) {  // K = 16 of the head dimension per step
+                  const uint32_t off = (kk >> 2) * (kAttnTileBytes / 2) + (kk & 3) * 32;
+                  umma_bf16(ts, sdesc_sw128(qa + off, 16, 1024), sdesc_sw128(kb + off, 16, 1024), id_s, kk > 0 ? 1u : 0u);
+                }
+                umma_commit(s_full + t);
+                if (j == nb[t] - 1) umma_commit(q_empty + t);  // Q may be replaced
               }
-              umma_commit(s_full + t);
+              __syncwarp();
               ++blk[t];
-              if (j == nb[t] - 1) umma_commit(q_empty + t);  // Q may be replaced
             }
           }
           if (!ok) break;
           if (j > 0) {
-            umma_commit(v_empty + vst);
+            if (elect_one()) umma_commit(v_empty + vst);
+            __syncwarp();
             if (++vst == kVStages) { vst = 0; vph ^= 1u; }
           }
           if (j < nkb) {
-            umma_commit(k_empty + st);
+            if (elect_one()) umma_commit(k_empty + st);
+            __syncwarp();
             if (++st == kKStages) { st = 0; ph ^= 1u; }
           }
         }
       }
-      umma_commit(drain);               // every issued MMA completes before TMEM is released
+      if (elect_one()) umma_commit(drain);               // every issued MMA completes before TMEM is released
       WaitCtx wd = wc;
       int dummy = 0;
       wd.abort_flag = &dummy;

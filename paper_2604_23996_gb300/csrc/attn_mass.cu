@@ -146,7 +146,7 @@ k_attn_mass(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
   volatile uint32_t* decision = reinterpret_cast<volatile uint32_t*>(tmem_slot + 2);   // [2]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int BH = p.B * p.H;
   const int n_items = ((p.n_qtiles + 1) / 2) * BH;
   WaitCtx wc{abort_flag, p.status, p.limit_ns};
@@ -186,7 +186,7 @@ k_attn_mass(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
+    {
       int st = 0;
       uint32_t ph = 0;
       int nqt[2] = {0, 0};              // items that used Q buffer t: its barrier phase
@@ -198,19 +198,25 @@ k_attn_mass(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         const Item w = decode_item(p, item);
         const int row0 = (w.b * p.H + w.h) * p.S;
         for (int t = 0; t < w.nq && ok; ++t) {
-          if (!mbar_wait(q_empty + t, (static_cast<uint32_t>(nqt[t]) & 1u) ^ 1u, wc)) { ok = false; break; }
+          if (!warp_wait(q_empty + t, (static_cast<uint32_t>(nqt[t]) & 1u) ^ 1u, wc)) { ok = false; break; }
           ++nqt[t];
-          mbar_arrive_expect_tx(q_full + t, kTile);
-          tma_load_2d(qs + t * kTile, &tmQ, q_full + t, 0, row0 + (w.qt0 + t) * kAT);
-          tma_load_2d(qs + t * kTile + kTile / 2, &tmQ, q_full + t, 64, row0 + (w.qt0 + t) * kAT);
+          if (elect_one()) {
+            mbar_arrive_expect_tx(q_full + t, kTile);
+            tma_load_2d(qs + t * kTile, &tmQ, q_full + t, 0, row0 + (w.qt0 + t) * kAT);
+            tma_load_2d(qs + t * kTile + kTile / 2, &tmQ, q_full + t, 64, row0 + (w.qt0 + t) * kAT);
+          }
+          __syncwarp();
         }
         const int nkb = kblocks_of(p, w.qt0 + w.nq - 1);
         for (int kb = 0; kb < nkb && ok; ++kb) {
-          if (!mbar_wait(kempty + st, ph ^ 1u, wc)) { ok = false; break; }
-          uint8_t* kd = ks + st * kTile;
-          mbar_arrive_expect_tx(kfull + st, kTile);
-          tma_load_2d(kd, &tmK, kfull + st, 0, row0 + kb * kAT);
-          tma_load_2d(kd + kTile / 2, &tmK, kfull + st, 64, row0 + kb * kAT);
+          if (!warp_wait(kempty + st, ph ^ 1u, wc)) { ok = false; break; }
+          if (elect_one()) {
+            uint8_t* kd = ks + st * kTile;
+            mbar_arrive_expect_tx(kfull + st, kTile);
+            tma_load_2d(kd, &tmK, kfull + st, 0, row0 + kb * kAT);
+            tma_load_2d(kd + kTile / 2, &tmK, kfull + st, 64, row0 + kb * kAT);
+          }
+          __syncwarp();
           ++issued;
           if (++st == n_ks) { st = 0; ph ^= 1u; }
         }
@@ -227,7 +233,7 @@ k_attn_mass(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16(kAT, kAT, false, false);
       int st = 0;
       uint32_t ph = 0;
@@ -239,41 +245,47 @@ k_attn_mass(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUt
         if (item >= n_items) break;
         const Item w = decode_item(p, item);
         for (int t = 0; t < w.nq && ok; ++t)
-          if (!mbar_wait(q_full + t, static_cast<uint32_t>(nqt[t]++) & 1u, wc)) ok = false;
+          if (!warp_wait(q_full + t, static_cast<uint32_t>(nqt[t]++) & 1u, wc)) ok = false;
         if (!ok) break;
         tc_fence_after();
         const int nkb0 = kblocks_of(p, w.qt0), nkb = kblocks_of(p, w.qt0 + w.nq - 1);
         for (int kb = 0; kb < nkb; ++kb) {
-          if (!mbar_wait(kfull + st, ph, wc)) { ok = false; break; }
+          if (!warp_wait(kfull + st, ph, wc)) { ok = false; break; }
           tc_fence_after();
           const uint32_t kbase = smem_u32(ks + st * kTile);
           for (int t = 0; t < w.nq; ++t) {
             if (t == 0 && kb >= nkb0) continue;       // past the first tile's diagonal
             const int buf = blk[t] & 1;
-            if (!mbar_wait(s_empty + 2 * t + buf, (static_cast<uint32_t>(blk[t] >> 1) & 1u) ^ 1u, wc)) {
+            if (!warp_wait(s_empty + 2 * t + buf, (static_cast<uint32_t>(blk[t] >> 1) & 1u) ^ 1u, wc)) {
               ok = false;
               break;
             }
             tc_fence_after();
             const uint32_t qa = smem_u32(qs + t * kTile);
             const uint32_t d_tmem = tmem + static_cast<uint32_t>((2 * t + buf) * kAT);
+            if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < kHd / 16; ++kk) {
-              const uint32_t off = (kk >> 2) * (kTile / 2) + (kk & 3) * 32;
-              umma_bf16(d_tmem, sdesc_sw128(qa + off, 16, 1024), sdesc_sw128(kbase + off, 16, 1024), idesc,
-                        kk > 0 ? 1u : 0u);
+              for (int kk = 0; kk < kHd / 16; ++kk) {
+                const uint32_t off = (kk >> 2) * (kTile / 2) + (kk & 3) * 32;
+                umma_bf16(d_tmem, sdesc_sw128(qa + off, 16, 1024), sdesc_sw128(kbase + off, 16, 1024), idesc,
+                          kk > 0 ? 1u : 0u);
+              }
+              umma_commit(s_full + 2 * t + buf);
             }
-            umma_commit(s_full + 2 * t + buf);
+            __syncwarp();
             ++blk[t];
           }
           if (!ok) break;
-          umma_commit(kempty + st);
+          if (elect_one()) umma_commit(kempty + st);
+          __syncwarp();
           if (++st == n_ks) { st = 0; ph ^= 1u; }
         }
         if (!ok) break;
-        for (int t = 0; t < w.nq; ++t) umma_commit(q_empty + t);   // Q tiles may be replaced
+        if (elect_one())
+          for (int t = 0; t < w.nq; ++t) umma_commit(q_empty + t); // Q tiles may be replaced
+        __syncwarp();
       }
-      umma_commit(drain);
+      if (elect_one()) umma_commit(drain);
       WaitCtx wd = wc;
       int dummy = 0;
       wd.abort_flag = &dummy;

@@ -85,6 +85,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   }
 }
 
+// The producer and MMA roles run their loops with the whole warp converged and issue through one
+// elected lane: TMA and tcgen05 instructions take their operands from uniform registers, which the
+// compiler fills directly when the warp is known to be converged. Under `if (lane == 0)` it moved
+// every operand there anew, about 85 cycles per tcgen05.mma against 64 of tensor time, and that
+// set the rate of the forward and of the backward.
+__device__ __forceinline__ int warp_index() {       // the same in every lane, and known to be
+  return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
+}
+__device__ __forceinline__ bool elect_one() {       // always the same lane
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, w));
+}
+
 // Grid barrier for co-resident blocks, called by one thread per block. sync[0] counts
 // arrivals, sync[1] is the generation; the last block resets the count and advances the
 // generation, so the pair is zero-count again between calls. A wait that exceeds limit_ns sets

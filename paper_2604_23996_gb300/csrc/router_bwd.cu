@@ -397,7 +397,7 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stg_full + kDrainGroups);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int S = p.slices, G = p.groups;
   const int sl = blockIdx.x % S, grp = blockIdx.x / S;
   const int d0 = sl * p.slice_width;
@@ -450,64 +450,69 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 
   if (warp == 0) {
     // -------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      bool ok = true;
-      int st = 0;
-      uint32_t ph = 0;
-      long issued = 0, dz_issued = 0;
-      int lt = 0;
-      for (int t = grp; t < p.n_tiles && ok; t += G, ++lt) {
-        const int zb = lt & 1;
-        const uint32_t zuse = static_cast<uint32_t>(lt >> 1);
-        if (!mbar_wait(dz_empty + zb, (zuse & 1u) ^ 1u, wc)) { ok = false; break; }
+    bool ok = true;
+    int st = 0;
+    uint32_t ph = 0;
+    long issued = 0, dz_issued = 0;
+    int lt = 0;
+    for (int t = grp; t < p.n_tiles && ok; t += G, ++lt) {
+      const int zb = lt & 1;
+      const uint32_t zuse = static_cast<uint32_t>(lt >> 1);
+      if (!warp_wait(dz_empty + zb, (zuse & 1u) ^ 1u, wc)) { ok = false; break; }
+      if (elect_one()) {
         mbar_arrive_expect_tx(dz_full + zb, dz_buf_bytes);
         bulk_load(dzb + zb * dz_buf_bytes, p.ws.dz_img + static_cast<size_t>(t) * dz_buf_bytes,
                   dz_buf_bytes, dz_full + zb);
-        ++dz_issued;
-        for (int b = 0; b < nb; ++b) {
-          if (!mbar_wait(xempty + st, ph ^ 1u, wc)) { ok = false; break; }
+      }
+      __syncwarp();
+      ++dz_issued;
+      for (int b = 0; b < nb; ++b) {
+        if (!warp_wait(xempty + st, ph ^ 1u, wc)) { ok = false; break; }
+        if (elect_one()) {
           uint8_t* xs = xst + st * 16384;
           mbar_arrive_expect_tx(xfull + st, 16384u);
           tma_load_2d(xs, &tmX, xfull + st, d0 + b * kBwdBD, t * kBwdBT);
           tma_load_2d(xs + 8192, &tmX, xfull + st, d0 + b * kBwdBD + 64, t * kBwdBT);
-          ++issued;
-          if (++st == n_xst) { st = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        ++issued;
+        if (++st == n_xst) { st = 0; ph ^= 1u; }
       }
-      WaitCtx wd = wc;
-      int dummy = 0;
-      wd.abort_flag = &dummy;
-      mbar_wait(wfull, 0, wd);                // the W slice copy must land before exit
-      if (!ok) {                              // so must every issued X and dz copy
-        for (long q = (issued > n_xst ? issued - n_xst : 0); q < issued; ++q)
-          mbar_wait(xfull + (q % n_xst), static_cast<uint32_t>((q / n_xst) & 1), wd);
-        for (long q = (dz_issued > 2 ? dz_issued - 2 : 0); q < dz_issued; ++q)
-          mbar_wait(dz_full + (q & 1), static_cast<uint32_t>((q >> 1) & 1), wd);
-      }
+    }
+    WaitCtx wd = wc;
+    int dummy = 0;
+    wd.abort_flag = &dummy;
+    mbar_wait(wfull, 0, wd);                  // the W slice copy must land before exit
+    if (!ok) {                                // so must every issued X and dz copy
+      for (long q = (issued > n_xst ? issued - n_xst : 0); q < issued; ++q)
+        mbar_wait(xfull + (q % n_xst), static_cast<uint32_t>((q / n_xst) & 1), wd);
+      for (long q = (dz_issued > 2 ? dz_issued - 2 : 0); q < dz_issued; ++q)
+        mbar_wait(dz_full + (q & 1), static_cast<uint32_t>((q >> 1) & 1), wd);
     }
   } else if (warp == 1) {
     // -------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t id_dw = idesc_bf16(128, E_pad, true, true);
-      const uint32_t id_dx = idesc_bf16(128, kBwdBT, true, false);
-      bool ok = mbar_wait(wfull, 0, wc);
+    const uint32_t id_dw = idesc_bf16(128, E_pad, true, true);
+    const uint32_t id_dx = idesc_bf16(128, kBwdBT, true, false);
+    const uint32_t dz0 = smem_u32(dzb), xst0 = smem_u32(xst), wsl0 = smem_u32(wsl);
+    bool ok = warp_wait(wfull, 0, wc);
+    tc_fence_after();
+    int st = 0;
+    uint32_t ph = 0;
+    int it = 0;                                // d-block iterations of this CTA
+    int lt = 0;
+    for (int t = grp; t < p.n_tiles && ok; t += G, ++lt) {
+      const int zb = lt & 1;
+      const uint32_t zuse = static_cast<uint32_t>(lt >> 1);
+      if (!warp_wait(dz_full + zb, zuse & 1u, wc)) { ok = false; break; }
       tc_fence_after();
-      int st = 0;
-      uint32_t ph = 0;
-      int it = 0;                              // d-block iterations of this CTA
-      int lt = 0;
-      for (int t = grp; t < p.n_tiles && ok; t += G, ++lt) {
-        const int zb = lt & 1;
-        const uint32_t zuse = static_cast<uint32_t>(lt >> 1);
-        if (!mbar_wait(dz_full + zb, zuse & 1u, wc)) { ok = false; break; }
+      const uint32_t hi = dz0 + static_cast<uint32_t>(zb) * dz_buf_bytes;
+      const uint32_t lo = hi + dz_half;
+      for (int b = 0; b < nb; ++b, ++it) {
+        if (!warp_wait(xfull + st, ph, wc)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t hi = smem_u32(dzb + zb * dz_buf_bytes);
-        const uint32_t lo = hi + dz_half;
-        for (int b = 0; b < nb; ++b, ++it) {
-          if (!mbar_wait(xfull + st, ph, wc)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t xs = smem_u32(xst + st * 16384);
-          const uint32_t dwc = tmem + static_cast<uint32_t>(b * E_pad);
+        const uint32_t xs = xst0 + static_cast<uint32_t>(st) * 16384u;
+        const uint32_t dwc = tmem + static_cast<uint32_t>(b * E_pad);
+        if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < kBwdBT / 16; ++ks) {     // K = 16 tokens per instruction
             const uint64_t da = sdesc_sw128(xs + ks * 2048, 8192, 1024);
@@ -517,14 +522,17 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             umma_bf16(dwc, da, dl, id_dw, 1u);
           }
           umma_commit(xempty + st);             // the X stage is free once these MMAs complete
-          if (++st == n_xst) { st = 0; ph ^= 1u; }
-          if (want_dx) {
-            const int xb = it % kDxBufs;
-            const uint32_t xuse = static_cast<uint32_t>(it / kDxBufs);
-            if (!mbar_wait(dx_empty + xb, (xuse & 1u) ^ 1u, wc)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t dxc = tm_dx + static_cast<uint32_t>(xb * kBwdBT);
-            const uint32_t wa = smem_u32(wsl + 2 * b * dz_half);
+        }
+        __syncwarp();
+        if (++st == n_xst) { st = 0; ph ^= 1u; }
+        if (want_dx) {
+          const int xb = it % kDxBufs;
+          const uint32_t xuse = static_cast<uint32_t>(it / kDxBufs);
+          if (!warp_wait(dx_empty + xb, (xuse & 1u) ^ 1u, wc)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t dxc = tm_dx + static_cast<uint32_t>(xb * kBwdBT);
+          const uint32_t wa = wsl0 + static_cast<uint32_t>(2 * b) * dz_half;
+          if (elect_one()) {
 #pragma unroll
             for (int ke = 0; ke < E_pad / 16; ++ke) {    // K = 16 experts per instruction
               const uint64_t da = sdesc_sw128(wa + ke * 2048, dz_half, 1024);
@@ -534,17 +542,22 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             }
             umma_commit(dx_full + xb);
           }
+          __syncwarp();
         }
-        if (!ok) break;
-        umma_commit(dz_empty + zb);
       }
+      if (!ok) break;
+      if (elect_one()) umma_commit(dz_empty + zb);
+      __syncwarp();
+    }
+    if (elect_one()) {
       if (ok) umma_commit(dw_full);
       umma_commit(drain);
-      WaitCtx wd = wc;
-      int dummy = 0;
-      wd.abort_flag = &dummy;
-      mbar_wait(drain, 0, wd);
     }
+    __syncwarp();
+    WaitCtx wd = wc;
+    int dummy = 0;
+    wd.abort_flag = &dummy;
+    mbar_wait(drain, 0, wd);
   } else {
     // -------------------------------------------------------------- dX drain + dW drain (2 groups)
     const int lg = warp & 3;                           // TMEM lane quarter of this warp
