@@ -104,6 +104,7 @@ Dims make_dims(const smoes_plan_s* P) {
   m.pstride = piece_stride(d.n_bins);
   m.n_groups = P->n_groups;
   m.contig_bins = P->contig_bins ? 1 : 0;
+  m.nb_mul = static_cast<uint32_t>((65536 + P->N_B - 1) / P->N_B);
   return m;
 }
 

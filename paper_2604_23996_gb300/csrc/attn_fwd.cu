@@ -98,13 +98,6 @@ __device__ __forceinline__ int kblocks_of(const AttnParams& p, int qt) {
   return p.causal ? min(qt + 1, nk) : nk;
 }
 
-// 16 bytes of shared memory as two pairs.
-__device__ __forceinline__ ulonglong2 lds128(uint32_t addr) {
-  ulonglong2 v;
-  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(addr));
-  return v;
-}
-
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -245,7 +238,7 @@ __device__ __forceinline__ HalfTerms half_terms(const float* stage, int kb, int 
   return HalfTerms{s + k0 * 4u, s + (kKtKeys + k0) * 4u, s + 2u * kKtKeys * 4u + k0 / 32u * 16u};
 }
 __device__ __forceinline__ KeyChunk key_chunk(const HalfTerms& h, int c) {
-  const ulonglong2 v = lds128(h.chunk + 16u * c);
+  const ulonglong2 v = lds_u64x2(h.chunk + 16u * c);
   KeyChunk k;
   k.bias = lo2(v.x);
   k.m = hi2(v.x);
@@ -273,7 +266,7 @@ __device__ __forceinline__ float load_scores(uint32_t ts, const HalfTerms& h, fl
     const uint64_t sc2 = pack2(sc, sc);
 #pragma unroll
     for (int i4 = 0; i4 < kHalf / 4; ++i4) {
-      const ulonglong2 bb = lds128(h.bias + 16u * i4);
+      const ulonglong2 bb = lds_u64x2(h.bias + 16u * i4);
       x[2 * i4] = ffma2(x[2 * i4], sc2, bb.x);
       x[2 * i4 + 1] = ffma2(x[2 * i4 + 1], sc2, bb.y);
     }
@@ -333,7 +326,7 @@ __device__ __forceinline__ void weigh(uint64_t (&x)[kHalf / 2], uint64_t f2, con
       uint64_t a0 = 0ull, a1 = 0ull;
 #pragma unroll
       for (int i4 = 0; i4 < 8; ++i4) {
-        const ulonglong2 mm = lds128(h.m + 16u * (c * 8 + i4));
+        const ulonglong2 mm = lds_u64x2(h.m + 16u * (c * 8 + i4));
         a0 = ffma2(x[16 * c + 2 * i4], mm.x, a0);
         a1 = ffma2(x[16 * c + 2 * i4 + 1], mm.y, a1);
       }

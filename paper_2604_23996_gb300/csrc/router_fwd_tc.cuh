@@ -31,6 +31,12 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kTileRows = kPieceTokens;      // 128 tokens per tile and per partial-sum piece
 constexpr int kPsStride = kTileRows + 1;     // padded row of the per-bin / per-modality tables
 constexpr int kMaxNV = piece_values(kMaxBins);
+// Bin of expert e under consecutive bins: e / N_B as a product (exact for e < 256: the error of
+// ceil(2^16 / N_B) adds less than 256 / 2^16 < 1 / N_B). A runtime division takes ~25 dependent
+// instructions, once per selected expert on the epilogue's latency chain.
+__device__ __forceinline__ int contig_bin(int e, uint32_t nb_mul) {
+  return static_cast<int>((static_cast<uint32_t>(e) * nb_mul) >> 16);
+}
 constexpr int kCoefBars = 8;                 // Gaussian coefficient chunks with their own barrier
 
 // Top-k selection key: the logit with its low `ib` mantissa bits replaced by the expert index,
@@ -247,6 +253,7 @@ struct EpiSmem {
   float* wpart;          // [2][4][kMaxNV] per-lane-quarter partial piece sums (double buffer)
   float* red;            // [kMaxNV] sample-reduce scratch of the first warp
   int* ctot;             // [kMaxBins] (token, bin) pairs of the CTA's tiles (fused permutation)
+  uint8_t* sel;          // [2 tiles][kMaxTopK][128] the rows' experts (fused permutation, <= 2 tiles)
   float* xmax;           // [2][128] per-group row maxima of the logits
   float* xsum;           // [2][128] per-group row sums of exp(z - max)
   float* xtk;            // [kMaxTopK][128] group 1's top-k keys of each row
@@ -263,9 +270,10 @@ struct EpiSmem {
   const CUtensorMap* tmG;
 };
 
+constexpr size_t kSelBytes = 2u * kMaxTopK * 128u;
 __host__ __device__ inline size_t epi_smem_floats(int K) {
   return static_cast<size_t>(K) * kPsStride + 5u * kPsStride + 2u * 4u * kMaxNV + kMaxNV + kMaxBins +
-         4u * 128u + static_cast<size_t>(kMaxTopK) * 128u;
+         4u * 128u + static_cast<size_t>(kMaxTopK) * 128u + kSelBytes / 4u;
 }
 
 __device__ inline EpiSmem epi_smem(float* base, int K, uint64_t* bars) {
@@ -278,6 +286,7 @@ __device__ inline EpiSmem epi_smem(float* base, int K, uint64_t* bars) {
   es.xmax = es.red + kMaxNV + kMaxBins;
   es.xsum = es.xmax + 256;
   es.xtk = es.xsum + 256;
+  es.sel = reinterpret_cast<uint8_t*>(es.xtk + kMaxTopK * 128);
   es.bar_in = bars;
   es.bar_out = bars + 1;
   es.xbar = bars + 2;
@@ -316,8 +325,9 @@ __device__ __forceinline__ int epi_split(const Dims& dm) {
 // the bin sums of e and the saved scores (e is saved with 1/sum kept per row, so that nothing
 // waits for the sum before storing). Group 0 then writes the top-k outputs and the permutation's
 // pair counts, group 1 the modality score; both write the per-(tile, sample) partial sums of the
-// joint table (eq. 12), each a half of the values. With the fused permutation, after the CTA's
-// last tile the first warp arrives on es.perm_go once all rows are counted.
+// joint table (eq. 12), each a half of the values. With the fused permutation, the first thread
+// arrives on es.perm_go as soon as the rows of the CTA's last tile are counted (the partial sums
+// and their fence follow).
 template <int KM, bool kVar, class Src, class Release>
 __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release& release, int tile,
                               int grp, int row, int lt, float dll, const TileMeta& meta,
@@ -520,7 +530,7 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
         for (int i = 0; i < KM; ++i) {
           if (i < k) {
             const int e = topk_index(tk[i], imask);
-            const int b = dm.contig_bins ? e / dm.N_B : __ldg(p.ws.expert_bin + e);
+            const int b = dm.contig_bins ? contig_bin(e, dm.nb_mul) : __ldg(p.ws.expert_bin + e);
             prow[b * kPsStride] += w[i] * iw;
           }
         }
@@ -535,7 +545,8 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
         for (int i = 0; i < KM; ++i) {
           if (i < k) {
             const int e = topk_index(tk[i], imask);
-            bins |= 1u << (dm.contig_bins ? e / dm.N_B : __ldg(p.ws.expert_bin + e));
+            es.sel[(lt * kMaxTopK + i) * 128 + row] = static_cast<uint8_t>(e);
+            bins |= 1u << (dm.contig_bins ? contig_bin(e, dm.nb_mul) : __ldg(p.ws.expert_bin + e));
           }
         }
       }
@@ -572,6 +583,8 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
   }
   mbar_arrive(es.xbar + 2);
   if (!mbar_wait(es.xbar + 2, xph, wc)) return;
+  // every row's selection and pair counts are in shared memory: the permutation's warps may go on
+  if (p.perm.perm_token && last_tile && grp == 0 && row == 0) mbar_arrive(es.perm_go);
   if (valid && p.bin_prob)
     for (int b = grp; b < K; b += 2) p.bin_prob[static_cast<size_t>(j) * K + b] = prow[b * kPsStride];
 
@@ -619,8 +632,6 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
     if (lane == 0) ok = mbar_wait(es.bar_out, static_cast<uint32_t>(lt & 1), wc);
     ok = __shfl_sync(0xffffffffu, ok, 0);
     if (!ok) return;
-    // every row of the CTA's last tile is done: its top-k and pair counts may be read
-    if (p.perm.perm_token && last_tile && lane == 0) mbar_arrive(es.perm_go);
     for (int s = s0; s <= s1; ++s) {
       // a sample strictly inside the tile has this tile's piece only
       const int pb = s == s0 ? meta.pb0 : s == s1 ? meta.pb1 : meta.pbase + (s - s0);
@@ -663,7 +674,8 @@ struct PermSel {
 };
 
 template <int KM>
-__device__ __forceinline__ void perm_load_sel(const FwdParams& p, int j, PermSel<KM>& t) {
+__device__ __forceinline__ void perm_load_sel(const FwdParams& p, const uint8_t* sel, int lt, int row, int j,
+                                              PermSel<KM>& t) {
   const Dims& dm = p.dm;
   const FusedPerm& f = p.perm;
   const bool valid = j < dm.T;
@@ -676,9 +688,9 @@ __device__ __forceinline__ void perm_load_sel(const FwdParams& p, int j, PermSel
     t.b[i] = -1;
     t.sbit[i] = 0u;
     if (valid && i < dm.k) {
-      const int e = __ldcg(p.topk_idx + static_cast<size_t>(j) * dm.k + i);   // this CTA's rows
+      const int e = sel[(lt * kMaxTopK + i) * 128 + row];
       t.e[i] = e;
-      t.b[i] = dm.contig_bins ? e / dm.N_B : __ldg(p.ws.expert_bin + e);
+      t.b[i] = dm.contig_bins ? contig_bin(e, dm.nb_mul) : __ldg(p.ws.expert_bin + e);
       t.sbit[i] = 1u << __ldg(p.ws.expert_slot + e);
       t.bins |= 1u << t.b[i];
     }
@@ -694,11 +706,12 @@ __device__ __forceinline__ void perm_load_sel(const FwdParams& p, int j, PermSel
 }
 
 // gtid: the thread's index in the group (0 .. 32 nw - 1); bar_id: a named barrier for the group;
-// ctot: the CTA's pair counts per bin (complete at perm_go); scratch: perm_scratch_ints(E) ints of
+// ctot, selb: the CTA's pair counts per bin and its rows' experts (complete at perm_go); scratch: perm_scratch_ints(E) ints of
 // shared memory that nothing else uses after perm_go.
 template <int KM>
 __device__ void perm_tail(const FwdParams& p, int t_beg, int t_end, int gtid, int nw, int bar_id,
-                          const int* ctot, int* scratch, uint64_t* perm_go, const WaitCtx& wc) {
+                          const int* ctot, const uint8_t* selb, int* scratch, uint64_t* perm_go,
+                          const WaitCtx& wc) {
   const Dims& dm = p.dm;
   const FusedPerm& f = p.perm;
   const int K = dm.K, E = dm.E;
@@ -716,7 +729,7 @@ __device__ void perm_tail(const FwdParams& p, int t_beg, int t_end, int gtid, in
   // the first round's selections (they land while the other CTAs finish), then the CTA's counts
   const int G = gridDim.x;
   PermSel<KM> sel;
-  perm_load_sel<KM>(p, t_beg * kTileRows + gtid, sel);
+  perm_load_sel<KM>(p, selb, 0, gtid, t_beg * kTileRows + gtid, sel);
   if (gtid < K) f.cta_counts[gtid * G + blockIdx.x] = ctot[gtid];
   for (int i = gtid; i < K * K; i += gs) disp[i] = 0;
   for (int i = gtid; i < 2 * E; i += gs) ecnt[i] = 0;
@@ -767,7 +780,7 @@ __device__ void perm_tail(const FwdParams& p, int t_beg, int t_end, int gtid, in
   for (int tile = t_beg; tile < t_end; ++tile) {
     for (int r0 = 0; r0 < kTileRows; r0 += gs) {
       const int j = tile * kTileRows + r0 + gtid;
-      if (!first) perm_load_sel<KM>(p, j, sel);
+      if (!first) perm_load_sel<KM>(p, selb, tile - t_beg, r0 + gtid, j, sel);
       first = false;
       for (int kb = 0; kb < K; ++kb) {
         const unsigned bal = __ballot_sync(0xffffffffu, (sel.bins >> kb) & 1u);
@@ -999,14 +1012,15 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       // the Gaussian statistics are requested before the X stream floods the memory system
       if (kGauss) ok = mbar_wait(coef_issued, 0, wc);
       for (int tile = t_beg; tile < t_end && ok; ++tile) {
+        int kx = kb0;
         for (int kb = 0; kb < n_kb; ++kb) {
           if (!mbar_wait(empty + st, ph ^ 1u, wc)) { ok = false; break; }
           uint8_t* xs = stage + st * sbytes;
           mbar_arrive_expect_tx(full + st, tx);
-          const int kx = kb_at(kb);
           tma_load_2d(xs, &tmX, full + st, kx * kFwdBK, tile * kFwdBM);
           tma_load_2d(xs + 16384, &tmW, full + st, kx * kFwdBK, 0);
           ++issued;
+          if (++kx == n_kb) kx = 0;
           if (++st == n_stages) { st = 0; ph ^= 1u; }
         }
       }
@@ -1132,14 +1146,19 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         uint64_t acc2[32];                   // per row: {sum over even features, over odd}
 #pragma unroll
         for (int r = 0; r < 32; ++r) acc2[r] = 0ull;
+        int kx = kb0;
+        bool ready = false;                  // the stage is known to have landed
         for (int kb = 0; kb < n_kb; ++kb) {
           // the coefficients of this block's chunk (complete for every later tile)
           if (lt == 0 && (kb & 7) == 0 && kb < 8 * kCoefBars &&
               !mbar_wait(coef_bar + (kb >> 3), 0, wc)) { ok = false; break; }
-          if (!mbar_wait(full + st, ph, wc)) { ok = false; break; }
+          if (!ready && !mbar_wait(full + st, ph, wc)) { ok = false; break; }
           const uint8_t* xs = stage + st * sbytes + gw * 32 * 128;
           // {a_2l, a_2l+1} and {b_2l, b_2l+1} of the float4 {ga, ga, gb, gb}
-          const ulonglong2 cf = reinterpret_cast<const ulonglong2*>(cq)[kb_at(kb) * 32 + lane];
+          const ulonglong2 cf = reinterpret_cast<const ulonglong2*>(cq)[kx * 32 + lane];
+          // the next stage is asked for before this one is worked on (the answer takes ~200 cycles)
+          const int nst = st + 1 == n_stages ? 0 : st + 1;
+          ready = mbar_test(full + nst, nst ? ph : ph ^ 1u);
 #pragma unroll
           for (int r = 0; r < 32; ++r) {
             const uint32_t u = *reinterpret_cast<const uint32_t*>(xs + r * 128 + ((chk ^ (r & 7)) << 4) + wcol);
@@ -1149,6 +1168,7 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(empty + st);
+          if (++kx == n_kb) kx = 0;
           if (++st == n_stages) { st = 0; ph ^= 1u; }
         }
         if (!ok) break;
@@ -1165,10 +1185,10 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   // once their part of the CTA's tiles is done; the stage buffers are free after perm_go
   if (p.perm.perm_token) {
     int* ps = reinterpret_cast<int*>(stage);
-    const int* ctot = epi_smem(epi, dm.K, ebars).ctot;
+    const EpiSmem es = epi_smem(epi, dm.K, ebars);
     if (kGauss && warp >= 6 && warp < 10)
-      perm_tail<KM>(p, t_beg, t_end, threadIdx.x - 192, 4, 1, ctot, ps, perm_go, wc);
-    if (!kGauss && warp < 2) perm_tail<KM>(p, t_beg, t_end, threadIdx.x, 2, 1, ctot, ps, perm_go, wc);
+      perm_tail<KM>(p, t_beg, t_end, threadIdx.x - 192, 4, 1, es.ctot, es.sel, ps, perm_go, wc);
+    if (!kGauss && warp < 2) perm_tail<KM>(p, t_beg, t_end, threadIdx.x, 2, 1, es.ctot, es.sel, ps, perm_go, wc);
   }
 
   // the role branches leave single lanes running on their own: the warp reconverges before

@@ -66,6 +66,7 @@ struct Dims {
   int pstride;               // piece_stride(K)
   int n_groups;              // ceil(T / 128): forward tiles = partial-sum groups
   int contig_bins;           // bin b holds experts [b N_B, (b+1) N_B) and N_B % 4 == 0
+  uint32_t nb_mul;           // ceil(2^16 / N_B): e / N_B == (e nb_mul) >> 16 for e < 256
 };
 
 // The bin permutation of the forward's own top-k, done inside the forward launch (Sec. 4.5);
