@@ -45,7 +45,8 @@ constexpr int kCoefBars = 8;                 // Gaussian coefficient chunks with
 // expert index. Keys compare with float min/max.
 __device__ __forceinline__ float topk_key(float z, int e, uint32_t imask) {
   const uint32_t u = __float_as_uint(z);
-  const uint32_t low = (u & 0x80000000u) ? static_cast<uint32_t>(e) : imask - static_cast<uint32_t>(e);
+  const uint32_t sign = static_cast<uint32_t>(static_cast<int32_t>(u) >> 31);
+  const uint32_t low = (static_cast<uint32_t>(e) ^ imask) ^ (sign & imask);   // imask - e, or e
   return __uint_as_float((u & ~imask) | low);
 }
 
@@ -59,12 +60,55 @@ __device__ __forceinline__ float topk_logit(float key, uint32_t imask) {
   return __uint_as_float((__float_as_uint(key) & ~imask) | ((imask + 1u) >> 1));
 }
 
-// Sorted (descending) insertion of key q into tk[0..KM): new[i] = max(tk[i], min(tk[i-1], q)).
-template <int KM>
-__device__ __forceinline__ void topk_push(float (&tk)[KM], float q) {
+// Length of the running top-k list: k rounded up to a power of two.
+__host__ __device__ constexpr int topk_len(int KM) { return KM <= 2 ? 2 : KM <= 4 ? 4 : KM <= 8 ? 8 : 16; }
+
+__device__ __forceinline__ void cmp_desc(float& a, float& b) {
+  const float hi = fmaxf(a, b);
+  b = fminf(a, b);
+  a = hi;
+}
+// Descending sort of L keys (Batcher's odd-even merge sort: 19 exchanges for eight).
+template <int L>
+__device__ __forceinline__ void sort_desc(float (&v)[L]) {
 #pragma unroll
-  for (int i = KM - 1; i > 0; --i) tk[i] = fmaxf(tk[i], fminf(tk[i - 1], q));
-  tk[0] = fmaxf(tk[0], q);
+  for (int p = 1; p < L; p *= 2) {
+#pragma unroll
+    for (int k = p; k >= 1; k /= 2) {
+#pragma unroll
+      for (int j = k % p; j + k < L; j += 2 * k) {
+#pragma unroll
+        for (int i = 0; i < k; ++i)
+          if (i + j + k < L && (i + j) / (2 * p) == (i + j + k) / (2 * p)) cmp_desc(v[i + j], v[i + j + k]);
+      }
+    }
+  }
+}
+// tk <- the L largest keys of tk and v, both descending: the larger of tk[i] and v[L-1-i] are those
+// L keys as a bitonic sequence, sorted by a bitonic merge. With the sort this takes 70 minima and
+// maxima per eight keys (L = 8), in short chains; inserting key by key took 15 per key in one chain.
+template <int L>
+__device__ __forceinline__ void topk_merge(float (&tk)[L], const float (&v)[L]) {
+#pragma unroll
+  for (int i = 0; i < L; ++i) tk[i] = fmaxf(tk[i], v[L - 1 - i]);
+#pragma unroll
+  for (int j = L / 2; j >= 1; j /= 2) {
+#pragma unroll
+    for (int i = 0; i < L; ++i)
+      if ((i & j) == 0) cmp_desc(tk[i], tk[i + j]);
+  }
+}
+// The keys of 16 logits (experts 16 c + t) into the running list.
+template <int L>
+__device__ __forceinline__ void topk_take16(float (&tk)[L], const float (&v)[16], int c, uint32_t imask) {
+#pragma unroll
+  for (int t0 = 0; t0 < 16; t0 += L) {
+    float q[L];
+#pragma unroll
+    for (int t = 0; t < L; ++t) q[t] = topk_key(v[t0 + t], c * 16 + t0 + t, imask);
+    sort_desc<L>(q);
+    topk_merge<L>(tk, q);
+  }
 }
 
 // Coefficients of the feature pair (2i, 2i+1) (eqs. 8-9) into shared memory as
@@ -112,21 +156,20 @@ __device__ __noinline__ void sample_reduce(const FwdParams& p, int s, float* red
   // lane l sums value 32c + l over the sample's pieces in piece order, 32 loads in flight (one
   // round of memory latency per 32 pieces: the reduction sits on the forward's tail)
 #pragma unroll 1
-  for (int c = 0; c * 32 < NV; ++c) {
-    const int v = 32 * c + lane;
-    const bool in = v < NV;
+  for (int c = 0; c * 32 < NV && !dry; ++c) {
+    const int v = min(32 * c + lane, NV - 1);
     float acc = 0.f;
 #pragma unroll 1
     for (int q0 = pb; q0 < pe; q0 += 32) {
-      const float* src = p.ws.pieces + static_cast<size_t>(q0) * dm.pstride + (in ? v : 0);
+      // (addresses clamped instead of loads skipped: a branch per load took 0.1 us each)
       float t[32];
 #pragma unroll
       for (int i = 0; i < 32; ++i)
-        t[i] = (in && !dry && q0 + i < pe) ? __ldcg(src + static_cast<size_t>(i) * dm.pstride) : 0.f;
+        t[i] = __ldcg(p.ws.pieces + static_cast<size_t>(min(q0 + i, pe - 1)) * dm.pstride + v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) acc += t[i];
+      for (int i = 0; i < 32; ++i) acc += q0 + i < pe ? t[i] : 0.f;
     }
-    if (in) red[v] = acc;
+    red[v] = acc;
   }
   __syncwarp();
   const bool act = lane < K;
@@ -346,57 +389,44 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
   const uint32_t imask = (1u << (32 - __clz(max(nch * 16 - 1, 1)))) - 1u;
   const uint32_t xph = static_cast<uint32_t>(lt & 1);
 
-  // pass A: row maximum and top-k keys of this group's columns, even and odd columns in two
-  // independent lists (two dependency chains), merged at the end
-  float tk[KM], tk2[KM];
+  // pass A: row maximum and top-k keys of this group's columns
+  constexpr int L = topk_len(KM);
+  float tk[L];
 #pragma unroll
-  for (int i = 0; i < KM; ++i) tk[i] = tk2[i] = -CUDART_INF_F;
+  for (int i = 0; i < L; ++i) tk[i] = -CUDART_INF_F;
   float mx = -CUDART_INF_F, mx2 = -CUDART_INF_F;
-  if (!v_gate) {
 #pragma unroll 1
-    for (int c = cb; c < ce; ++c) {
-      float v[16];
-      src.load16(c, v);
+  for (int c = cb; c < ce; ++c) {
+    float v[16];
+    src.load16(c, v);
 #pragma unroll
-      for (int t = 0; t < 16; t += 2) {
-        mx = fmaxf(mx, v[t]);
-        mx2 = fmaxf(mx2, v[t + 1]);
-        topk_push<KM>(tk, topk_key(v[t], c * 16 + t, imask));
-        topk_push<KM>(tk2, topk_key(v[t + 1], c * 16 + t + 1, imask));
-      }
+    for (int t = 0; t < 16; t += 2) {
+      mx = fmaxf(mx, v[t]);
+      mx2 = fmaxf(mx2, v[t + 1]);
     }
-  } else {                           // sigmoid gate: the choice ranks s + bias (padding stays last)
-#pragma unroll 1
-    for (int c = cb; c < ce; ++c) {
-      float v[16];
-      src.load16(c, v);
+    if (v_gate) {                    // sigmoid gate: the choice ranks s + bias (padding stays last)
 #pragma unroll
       for (int t = 0; t < 16; ++t) {
         const int e = c * 16 + t;
-        mx = fmaxf(mx, v[t]);
         v[t] = e < E ? sigmoid_acc(v[t]) + (p.score_bias ? __ldg(p.score_bias + e) : 0.f) : -FLT_MAX;
       }
-#pragma unroll
-      for (int t = 0; t < 16; t += 2) {
-        topk_push<KM>(tk, topk_key(v[t], c * 16 + t, imask));
-        topk_push<KM>(tk2, topk_key(v[t + 1], c * 16 + t + 1, imask));
-      }
     }
+    topk_take16<L>(tk, v, c, imask);
   }
   mx = fmaxf(mx, mx2);
-#pragma unroll
-  for (int i = 0; i < KM; ++i) topk_push<KM>(tk, tk2[i]);
   es.xmax[grp * 128 + row] = mx;
   if (grp == 1 && split) {
 #pragma unroll
-    for (int i = 0; i < KM; ++i) es.xtk[i * 128 + row] = tk[i];
+    for (int i = 0; i < L; ++i) es.xtk[i * 128 + row] = tk[i];
   }
   mbar_arrive(es.xbar + 0);
   if (!mbar_wait(es.xbar + 0, xph, wc)) return;
   mx = fmaxf(es.xmax[row], es.xmax[128 + row]);
   if (grp == 0 && split) {
+    float o[L];
 #pragma unroll
-    for (int i = 0; i < KM; ++i) topk_push<KM>(tk, es.xtk[i * 128 + row]);
+    for (int i = 0; i < L; ++i) o[i] = es.xtk[i * 128 + row];
+    topk_merge<L>(tk, o);
   }
 
   // pass B: e = exp(z - max), its sum, the bin sums of e and the saved scores
@@ -602,16 +632,27 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
     const int r0 = 32 * wg + (mine ? __ffs(mine) - 1 : 0);
     const int r1 = 32 * wg + (mine ? 32 - __clz(mine) : 0);
     float* wp = es.wpart + ((n_in & 1) * 4 + wg) * kMaxNV;
-    for (int v = vb + lane; v < ve; v += 32) {
-      // value v: kind v / K over bin v % K (kind 0: Q, 1..4: weighted by m_s rows 0..3),
-      // or, past 5K, the plain sum of m_s row v - 5K
-      const int kind = v < 5 * K ? v / K : 0;
-      const float* a = v < 5 * K ? es.p_s + (v - kind * K) * kPsStride : es.m_s + (v - 5 * K) * kPsStride;
-      const float* w = es.m_s + (v < 5 * K ? (kind + 4) % 5 : 4) * kPsStride;
-      float acc = 0.f;
-#pragma unroll 4
-      for (int r = r0; r < r1; ++r) acc = fmaf(w[r], a[r], acc);
-      wp[v] = acc;
+    // value v: kind v / K over bin v % K (kind 0: Q, 1..4: weighted by m_s rows 0..3), or, past 5K,
+    // the plain sum of m_s row v - 5K; a thread forms two values in one walk over the rows, eight
+    // rows of loads in flight (one value at a time was the longest step of a tile with 16 bins)
+    for (int v0 = vb + lane; v0 < ve; v0 += 64) {
+      const float* a[2];
+      const float* w[2];
+      float acc[2] = {0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int v = min(v0 + 32 * q, ve - 1);
+        const int kind = v < 5 * K ? v / K : 0;
+        a[q] = v < 5 * K ? es.p_s + (v - kind * K) * kPsStride : es.m_s + (v - 5 * K) * kPsStride;
+        w[q] = es.m_s + (v < 5 * K ? (kind + 4) % 5 : 4) * kPsStride;
+      }
+#pragma unroll 8
+      for (int r = r0; r < r1; ++r) {
+        acc[0] = fmaf(w[0][r], a[0][r], acc[0]);
+        acc[1] = fmaf(w[1][r], a[1][r], acc[1]);
+      }
+      wp[v0] = acc[0];
+      if (v0 + 32 < ve) wp[v0 + 32] = acc[1];
     }
     mbar_arrive(es.bar_in);
     if (!mbar_wait(es.bar_in, n_in & 1u, wc)) return;
