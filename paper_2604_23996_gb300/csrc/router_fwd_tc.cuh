@@ -934,7 +934,7 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q); q += 4;
   int* abort_flag = reinterpret_cast<int*>(q);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   WaitCtx wc{abort_flag, p.ws.status, p.limit_ns};
 
   if (threadIdx.x == 0) {
@@ -1044,69 +1044,72 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      int st = 0;
-      uint32_t ph = 0;
-      long issued = 0;
-      bool ok = true;
-      const uint32_t tx = static_cast<uint32_t>(sbytes);
-      // the Gaussian statistics are requested before the X stream floods the memory system
-      if (kGauss) ok = mbar_wait(coef_issued, 0, wc);
-      for (int tile = t_beg; tile < t_end && ok; ++tile) {
-        int kx = kb0;
-        for (int kb = 0; kb < n_kb; ++kb) {
-          if (!mbar_wait(empty + st, ph ^ 1u, wc)) { ok = false; break; }
+    int st = 0;
+    uint32_t ph = 0;
+    long issued = 0;
+    const uint32_t tx = static_cast<uint32_t>(sbytes);
+    // the Gaussian statistics are requested before the X stream floods the memory system
+    bool ok = !kGauss || warp_wait(coef_issued, 0, wc);
+    for (int tile = t_beg; tile < t_end && ok; ++tile) {
+      int kx = kb0;
+      for (int kb = 0; kb < n_kb; ++kb) {
+        if (!warp_wait(empty + st, ph ^ 1u, wc)) { ok = false; break; }
+        if (elect_one()) {
           uint8_t* xs = stage + st * sbytes;
           mbar_arrive_expect_tx(full + st, tx);
           tma_load_2d(xs, &tmX, full + st, kx * kFwdBK, tile * kFwdBM);
           tma_load_2d(xs + 16384, &tmW, full + st, kx * kFwdBK, 0);
-          ++issued;
-          if (++kx == n_kb) kx = 0;
-          if (++st == n_stages) { st = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        ++issued;
+        if (++kx == n_kb) kx = 0;
+        if (++st == n_stages) { st = 0; ph ^= 1u; }
       }
-      if (!ok) {            // every issued copy must land before the CTA may exit
-        WaitCtx wd = wc;
-        int dummy = 0;
-        wd.abort_flag = &dummy;
-        for (long qn = (issued > n_stages ? issued - n_stages : 0); qn < issued; ++qn)
-          mbar_wait(full + (qn % n_stages), static_cast<uint32_t>((qn / n_stages) & 1), wd);
-      }
+    }
+    if (!ok) {              // every issued copy must land before the CTA may exit
+      WaitCtx wd = wc;
+      int dummy = 0;
+      wd.abort_flag = &dummy;
+      for (long qn = (issued > n_stages ? issued - n_stages : 0); qn < issued; ++qn)
+        mbar_wait(full + (qn % n_stages), static_cast<uint32_t>((qn / n_stages) & 1), wd);
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(kFwdBM, N, false, false);
-      int st = 0;
-      uint32_t ph = 0;
-      int lt = 0;
-      bool ok = true;
-      for (int tile = t_beg; tile < t_end && ok; ++tile, ++lt) {
-        const int buf = lt & 1;
-        const uint32_t use = static_cast<uint32_t>(lt >> 1);
-        if (!mbar_wait(acc_empty + buf, (use & 1u) ^ 1u, wc)) { ok = false; break; }
+    const uint32_t idesc = idesc_bf16(kFwdBM, N, false, false);
+    const uint32_t stage0 = smem_u32(stage), sbytes32 = static_cast<uint32_t>(sbytes);
+    int st = 0;
+    uint32_t ph = 0;
+    int lt = 0;
+    bool ok = true;
+    for (int tile = t_beg; tile < t_end && ok; ++tile, ++lt) {
+      const int buf = lt & 1;
+      const uint32_t use = static_cast<uint32_t>(lt >> 1);
+      if (!warp_wait(acc_empty + buf, (use & 1u) ^ 1u, wc)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * N);
+      for (int kb = 0; kb < n_kb; ++kb) {
+        if (!warp_wait(full + st, ph, wc)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(buf * N);
-        for (int kb = 0; kb < n_kb; ++kb) {
-          if (!mbar_wait(full + st, ph, wc)) { ok = false; break; }
-          tc_fence_after();
-          const uint8_t* xs = stage + st * sbytes;
-          const uint64_t da = sdesc_sw128(smem_u32(xs), 16, 1024);
-          const uint64_t db = sdesc_sw128(smem_u32(xs + 16384), 16, 1024);
+        const uint32_t xs = stage0 + static_cast<uint32_t>(st) * sbytes32;
+        const uint64_t da = sdesc_sw128(xs, 16, 1024);
+        const uint64_t db = sdesc_sw128(xs + 16384u, 16, 1024);
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < kFwdBK / 16; ++kk)   // K = 16 per instruction: +32 bytes
             umma_bf16(d_tmem, da + 2u * kk, db + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
           umma_commit(empty + st);
-          if (++st == n_stages) { st = 0; ph ^= 1u; }
+          if (kb == n_kb - 1) umma_commit(acc_full + buf);
         }
-        if (ok) umma_commit(acc_full + buf);
+        __syncwarp();
+        if (++st == n_stages) { st = 0; ph ^= 1u; }
       }
-      umma_commit(drain);   // every issued MMA completes before TMEM is released
-      WaitCtx wd = wc;
-      int dummy = 0;
-      wd.abort_flag = &dummy;
-      mbar_wait(drain, 0, wd);
     }
+    if (elect_one()) umma_commit(drain);   // every issued MMA completes before TMEM is released
+    __syncwarp();
+    WaitCtx wd = wc;
+    int dummy = 0;
+    wd.abort_flag = &dummy;
+    mbar_wait(drain, 0, wd);
   } else if (warp < 6 || warp >= (kGauss ? 10 : 6)) {
     // ---------------------------------------------------------------- epilogue (2 x 4 warps)
     const int grp = warp < 6 ? 0 : 1;        // column half of the logits
