@@ -698,7 +698,7 @@ smoes_status smoes_router_bwd(smoes_plan P, const void* X, const void* W, const 
         !encode_bf16_2d(&tw, W, d.E, d.d, E_pad, 64, true))
       return SMOES_ERR_CUDA;
     if (dX) {
-      if (!encode_bf16_2d(&tdx, dX, d.T, d.d, kBwdBT, kBwdBD, false)) return SMOES_ERR_CUDA;
+      if (!encode_bf16_2d(&tdx, dX, d.T, d.d, kBwdBT, 64, true)) return SMOES_ERR_CUDA;
     } else {
       tdx = tx;   // unused
     }

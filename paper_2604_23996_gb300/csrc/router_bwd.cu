@@ -342,6 +342,12 @@ __global__ void __launch_bounds__(256) k_dz_prep(const BwdParams p) {
 
 // ------------------------------------------------------------------ tcgen05 backward (bf16)
 
+__device__ __forceinline__ uint32_t cvt_pair(uint32_t lo, uint32_t hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
+  return d;
+}
+
 struct BwdLayout {
   uint32_t wsl, dz, xst, stg, bars, total;
 };
@@ -358,7 +364,7 @@ __host__ __device__ inline BwdLayout bwd_layout(int E_pad, int n_xst) {
   L.wsl = o;  o += 65536u;                                         // W slice (ds * E_pad * 2 B)
   L.dz = o;   o += 2u * 2u * static_cast<uint32_t>(E_pad) * 128u;   // 2 buffers x (hi, lo)
   L.xst = o;  o += static_cast<uint32_t>(n_xst) * 16384u;          // X stages [2 atoms][64][128 B]
-  L.stg = o;  o += kDrainGroups * 16384u;                          // dX staging [64][128] bf16 per group
+  L.stg = o;  o += kDrainGroups * 16384u;                          // dX staging [2 atoms][64][128 B] per group
   L.bars = o; o += 8u * (2u * n_xst + 32u) + 16u;
   L.total = o + 1024u;
   return L;
@@ -565,6 +571,12 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const int gtid = (threadIdx.x - 64) & 127;         // 0..127 within the group
     const bool issuer = (gtid == 0);
     uint8_t* sgb = stg + dg * 16384;
+    // matrix store addresses: lane 8 m + i gives row i (a token) of matrix m: tokens +8 for m / 2,
+    // d columns +8 for m % 2; the warp's d rows lie in atom lg / 2 from 16-byte chunk 4 (lg % 2)
+    const uint32_t st_row = static_cast<uint32_t>(lane & 7);
+    const uint32_t st_addr = smem_u32(sgb) + static_cast<uint32_t>(lg >> 1) * 8192u +
+                             static_cast<uint32_t>(lane >> 4) * 1024u + st_row * 128u;
+    const uint32_t st_chunk = 4u * static_cast<uint32_t>(lg & 1) + static_cast<uint32_t>((lane >> 3) & 1);
     bool ok = true;
     if (want_dx) {
       int it = 0, n_mine = 0;
@@ -580,15 +592,21 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
             mbar_arrive(stg_free + dg);
           }
           if (!mbar_wait(stg_free + dg, static_cast<uint32_t>(n_mine & 1), wc)) { ok = false; break; }
-          __nv_bfloat16* sg = reinterpret_cast<__nv_bfloat16*>(sgb);
+          // the warp's 32 d rows x 64 tokens to the staging's token rows (two swizzled 64-column
+          // atoms): 16-lane fragments whose register pairs are two tokens of a d row, packed to
+          // bf16 and stored transposed, eight 8 x 8 matrices of 16-byte rows at a time. A 2-byte
+          // store per element (64 per thread, against eight matrix stores) made this drain longer
+          // than the tile's MMAs.
           const uint32_t ta = tm_dx + (static_cast<uint32_t>(lg * 32) << 16) + static_cast<uint32_t>(xb * kBwdBT);
-          const int drow = lg * 32 + lane;
 #pragma unroll
-          for (int c = 0; c < kBwdBT / 32; ++c) {
-            float v[32];
-            tmem_ld32(ta + 32u * c, v);
+          for (int h = 0; h < 2; ++h) {                // d rows 16 h .. of the warp's 32
+            uint32_t r[32];
+            tmem_ld_16x256b_x8(ta + (static_cast<uint32_t>(16 * h) << 16), r);
 #pragma unroll
-            for (int q = 0; q < 32; ++q) sg[(c * 32 + q) * kBwdBD + drow] = __float2bfloat16_rn(v[q]);
+            for (int n = 0; n < 4; ++n)                // tokens 16 n .. 16 n + 15
+              stmatrix_x4_trans(st_addr + (((st_chunk + 2u * h) ^ st_row) << 4) + 2048u * n,
+                                cvt_pair(r[8 * n], r[8 * n + 1]), cvt_pair(r[8 * n + 2], r[8 * n + 3]),
+                                cvt_pair(r[8 * n + 4], r[8 * n + 5]), cvt_pair(r[8 * n + 6], r[8 * n + 7]));
           }
           tc_fence_before();
           mbar_arrive(dx_empty + xb);
@@ -596,7 +614,9 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           mbar_arrive(stg_full + dg);
           if (issuer) {
             if (!mbar_wait(stg_full + dg, static_cast<uint32_t>(n_mine & 1), wc)) { ok = false; break; }
-            tma_store_2d(&tmDX, sg, d0 + b * kBwdBD, t * kBwdBT);
+            const int dc = d0 + b * kBwdBD;
+            tma_store_2d(&tmDX, sgb, dc, t * kBwdBT);
+            if (dc + 64 < dm.d) tma_store_2d(&tmDX, sgb + 8192, dc + 64, t * kBwdBT);
             tma_store_commit();
           }
           ++n_mine;
