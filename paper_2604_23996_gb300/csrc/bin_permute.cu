@@ -21,37 +21,44 @@ namespace {
 constexpr int kPermThreads = 256;                    // one token per thread and round
 constexpr int kPermWarps = kPermThreads / 32;
 
-// One token's selection: its chosen experts (-1 for none) with their bins and slot bits, the
-// set of the bins and the token's modality (0 vision, 1 text). KM >= k, a compile-time bound
-// that keeps the arrays in registers.
+// One token's selection: the set of its chosen experts at position bin * N_B + slot of a 128-bit
+// set (plans hold at most 128 experts), so that a bin's mask is N_B consecutive bits, its experts in
+// bytes (0xff: none) for the counts, and its modality (0 vision, 1 text). Bins, slots and masks per
+// selected expert in registers of their own took 96 registers at k = 8: two blocks per SM, and two
+// rounds for 131072 tokens.
+constexpr int kSetWords = kMaxExpertsBf16 / 32;
 template <int KM>
 struct TokenSel {
-  int e[KM];
-  int b[KM];
-  uint32_t sbit[KM];
-  uint32_t bins;
+  uint32_t set[kSetWords];
+  uint32_t e4[(KM + 3) / 4];
   int m;
 };
 
 template <int KM>
-__device__ __forceinline__ void load_sel(const PermParams& p, const int* s_bin, const int* s_slot,
-                                         int j, TokenSel<KM>& s) {
-  s.bins = 0u;
+__device__ __forceinline__ void empty_sel(TokenSel<KM>& s) {
+#pragma unroll
+  for (int w = 0; w < kSetWords; ++w) s.set[w] = 0u;
+#pragma unroll
+  for (int q = 0; q < (KM + 3) / 4; ++q) s.e4[q] = 0xffffffffu;
+  s.m = 0;
+}
+
+template <int KM>
+__device__ __forceinline__ void load_sel(const PermParams& p, const uint8_t* s_pos, int j, TokenSel<KM>& s) {
+  empty_sel<KM>(s);
   int e[KM];
 #pragma unroll
   for (int i = 0; i < KM; ++i) e[i] = i < p.k ? p.topk_idx[static_cast<size_t>(j) * p.k + i] : -1;
   s.m = (p.is_vision && !p.is_vision[j]) ? 1 : 0;
 #pragma unroll
   for (int i = 0; i < KM; ++i) {
-    s.e[i] = -1;
-    s.b[i] = -1;
-    s.sbit[i] = 0u;
     if (i < p.k) {
       if (e[i] >= 0 && e[i] < p.E) {
-        s.e[i] = e[i];
-        s.b[i] = s_bin[e[i]];
-        s.sbit[i] = 1u << s_slot[e[i]];
-        s.bins |= 1u << s.b[i];
+        const uint32_t pos = s_pos[e[i]];
+        const uint32_t bit = 1u << (pos & 31u);
+#pragma unroll
+        for (int w = 0; w < kSetWords; ++w) s.set[w] |= (pos >> 5) == static_cast<uint32_t>(w) ? bit : 0u;
+        s.e4[i >> 2] ^= (0xffu ^ static_cast<uint32_t>(e[i])) << (8 * (i & 3));
       } else {
         atomicOr(p.status, kStatusData);
       }
@@ -59,10 +66,17 @@ __device__ __forceinline__ void load_sel(const PermParams& p, const int* s_bin, 
   }
 }
 
+// The first bin's mask of a set; the set then moves on to the next bin.
+__device__ __forceinline__ uint32_t next_mask(uint32_t (&set)[kSetWords], int NB, uint32_t nb_mask) {
+  const uint32_t m = set[0] & nb_mask;
+#pragma unroll
+  for (int w = 0; w < kSetWords; ++w) set[w] = __funnelshift_rc(set[w], w + 1 < kSetWords ? set[w + 1] : 0u, NB);
+  return m;
+}
+
 template <int KM>
 __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
-  __shared__ int s_bin[kMaxExperts];
-  __shared__ int s_slot[kMaxExperts];
+  __shared__ uint8_t s_pos[kMaxExperts];
   __shared__ int wcnt[kPermWarps][kMaxBins];
   __shared__ int base[kMaxBins];
   __shared__ int pre_s[kMaxBins], tot_s[kMaxBins];
@@ -74,11 +88,9 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
   pdl_wait();
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int K = p.K;
-  for (int e = threadIdx.x; e < p.E; e += kPermThreads) {
-    s_bin[e] = p.expert_bin[e];
-    s_slot[e] = p.expert_slot[e];
-  }
+  const int K = p.K, NB = p.E / p.K;
+  const uint32_t nb_mask = NB >= 32 ? 0xffffffffu : (1u << NB) - 1u;
+  for (int e = threadIdx.x; e < p.E; e += kPermThreads) s_pos[e] = static_cast<uint8_t>(p.expert_bin[e] * NB + p.expert_slot[e]);
   for (int i = threadIdx.x; i < K * K; i += kPermThreads) disp[i] = 0;
   for (int i = threadIdx.x; i < 2 * p.E; i += kPermThreads) ecnt[i] = 0;
   __syncthreads();
@@ -87,17 +99,15 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
   // selections stay in registers for the scatter
   int cnt = 0;
   TokenSel<KM> s0;
-  s0.bins = 0u;
-  s0.m = 0;
+  empty_sel<KM>(s0);
   for (int r = 0; r < p.rounds; ++r) {
     const int j = (blockIdx.x * p.rounds + r) * kPermThreads + threadIdx.x;
     TokenSel<KM> s;
-    s.bins = 0u;
-    s.m = 0;
-    if (j < p.T) load_sel<KM>(p, s_bin, s_slot, j, s);
+    empty_sel<KM>(s);
+    if (j < p.T) load_sel<KM>(p, s_pos, j, s);
     if (r == 0) s0 = s;
     for (int kb = 0; kb < K; ++kb) {
-      const int c = __popc(__ballot_sync(0xffffffffu, (s.bins >> kb) & 1u));
+      const int c = __popc(__ballot_sync(0xffffffffu, next_mask(s.set, NB, nb_mask) != 0u));
       if (lane == kb) cnt += c;
     }
   }
@@ -118,40 +128,48 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
   __syncthreads();
   if (!ok_s) return;
 
-  // offsets: warp w sums bins w, w + 8, ... over all blocks (lanes stride the blocks, eight
-  // loads in flight per lane and round)
+  // offsets: warp w sums bins w, w + 8, ... over all blocks (lanes stride the blocks, eight loads in
+  // flight per lane)
   for (int kb = warp; kb < K; kb += kPermWarps) {
     int pre = 0, tot = 0;
     const int* row = p.blk_counts + kb * p.n_blocks;
-    for (int b0 = lane; b0 < p.n_blocks; b0 += 8 * 32) {
+    int b0 = lane;
+    for (; b0 + 7 * 32 < p.n_blocks; b0 += 8 * 32) {
       int c[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) c[u] = b0 + 32 * u < p.n_blocks ? __ldcg(row + b0 + 32 * u) : 0;
+      for (int u = 0; u < 8; ++u) c[u] = __ldcg(row + b0 + 32 * u);
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         tot += c[u];
-        if (b0 + 32 * u < static_cast<int>(blockIdx.x)) pre += c[u];
+        pre += b0 + 32 * u < static_cast<int>(blockIdx.x) ? c[u] : 0;
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      pre += __shfl_xor_sync(0xffffffffu, pre, o);
-      tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    for (; b0 < p.n_blocks; b0 += 32) {
+      const int c = __ldcg(row + b0);
+      tot += c;
+      pre += b0 < static_cast<int>(blockIdx.x) ? c : 0;
     }
+    pre = __reduce_add_sync(0xffffffffu, pre);
+    tot = __reduce_add_sync(0xffffffffu, tot);
     if (lane == 0) {
       pre_s[kb] = pre;
       tot_s[kb] = tot;
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int kb = 0; kb < K; ++kb) {
-      base[kb] = run + pre_s[kb];
-      if (blockIdx.x == 0) p.bin_offsets[kb] = run;
-      run += tot_s[kb];
+  if (warp == 0) {                                      // bin bases: exclusive scan over the bins
+    const int t = lane < K ? tot_s[lane] : 0;
+    int run = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += v;
     }
-    if (blockIdx.x == 0) p.bin_offsets[K] = run;
+    if (lane < K) {
+      base[lane] = run - t + pre_s[lane];
+      if (blockIdx.x == 0) p.bin_offsets[lane] = run - t;
+      if (blockIdx.x == 0 && lane == K - 1) p.bin_offsets[K] = run;
+    }
   }
   __syncthreads();
 
@@ -160,14 +178,6 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
   for (int r = 0; r < p.rounds; ++r) {
     const int j = (blockIdx.x * p.rounds + r) * kPermThreads + threadIdx.x;
     const bool valid = j < p.T;
-    TokenSel<KM> s;
-    s.bins = 0u;
-    s.m = 0;
-    if (r == 0) {
-      s = s0;
-    } else if (valid) {
-      load_sel<KM>(p, s_bin, s_slot, j, s);
-    }
     int home = 0;
     if (valid) {
       home = p.home ? p.home[j] : static_cast<int>((static_cast<long long>(j) * K) / p.T);
@@ -176,11 +186,23 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
         home = -1;
       }
     }
-    for (int kb = 0; kb < K; ++kb) {
-      const unsigned bal = __ballot_sync(0xffffffffu, (s.bins >> kb) & 1u);
-      if (lane == 0) wcnt[warp][kb] = __popc(bal);
+    TokenSel<KM> s;
+    if (r == 0) {
+      s = s0;
+    } else {
+      empty_sel<KM>(s);
+      if (valid) load_sel<KM>(p, s_pos, j, s);
     }
-    __syncthreads();
+    if (p.rounds > 1) {                                 // (one round: wcnt still holds the warps' counts)
+      uint32_t set[kSetWords];
+#pragma unroll
+      for (int w = 0; w < kSetWords; ++w) set[w] = s.set[w];
+      for (int kb = 0; kb < K; ++kb) {
+        const unsigned bal = __ballot_sync(0xffffffffu, next_mask(set, NB, nb_mask) != 0u);
+        if (lane == 0) wcnt[warp][kb] = __popc(bal);
+      }
+      __syncthreads();
+    }
     if (threadIdx.x < K) {                              // exclusive scan over warps, per bin
       int run = base[threadIdx.x];
       for (int w = 0; w < kPermWarps; ++w) {
@@ -194,12 +216,10 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
     // lanes with the same dispatch home add their pairs with one atomic per (warp, bin, home)
     const unsigned same_home = __match_any_sync(0xffffffffu, home);
     for (int kb = 0; kb < K; ++kb) {
-      const unsigned bal = __ballot_sync(0xffffffffu, (s.bins >> kb) & 1u);
-      if ((s.bins >> kb) & 1u) {
+      const uint32_t mask = next_mask(s.set, NB, nb_mask);
+      const unsigned bal = __ballot_sync(0xffffffffu, mask != 0u);
+      if (mask) {
         const int pos = wcnt[warp][kb] + __popc(bal & lt_mask);
-        uint32_t mask = 0u;
-#pragma unroll
-        for (int i = 0; i < KM; ++i) mask |= (s.b[i] == kb) ? s.sbit[i] : 0u;
         p.perm_token[pos] = j;
         p.perm_mask[pos] = mask;
         const unsigned grp = bal & same_home;
@@ -208,8 +228,10 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
     }
     if (valid && p.expert_counts) {
 #pragma unroll
-      for (int i = 0; i < KM; ++i)
-        if (s.e[i] >= 0) atomicAdd(&ecnt[s.m * p.E + s.e[i]], 1);
+      for (int i = 0; i < KM; ++i) {
+        const uint32_t e = (s.e4[i >> 2] >> (8 * (i & 3))) & 0xffu;
+        if (e != 0xffu) atomicAdd(&ecnt[s.m * p.E + static_cast<int>(e)], 1);
+      }
     }
     __syncthreads();                                    // wcnt reused by the next round
   }
