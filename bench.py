@@ -213,7 +213,7 @@ class ClockSampler:
 
 # the sources whose code a call's kernels are compiled from (a traffic record counts only for them)
 TRAFFIC_SOURCES = {
-    "fwd": ["router_fwd.cu", "router_fwd_tc.cuh", "router_fwd_var.cu", "ptx.cuh", "device_common.cuh",
+    "fwd": ["router_fwd.cu", "router_fwd_tc.cuh", "router_fwd_f32.cuh", "router_fwd_var.cu", "ptx.cuh", "device_common.cuh",
             "smoes_internal.cuh"],
     "bwd": ["router_bwd.cu", "ptx.cuh", "device_common.cuh", "smoes_internal.cuh"],
 }

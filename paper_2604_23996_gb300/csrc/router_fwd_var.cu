@@ -1,7 +1,7 @@
-// router_fwd_var.cu -- the tensor-core router forward with the router variants compiled in
-// (sigmoid gate with a selection bias, top-k-masked bin sums of eq. (12)); the kernel and its
-// epilogue are in router_fwd_tc.cuh.
-#include "router_fwd_tc.cuh"
+// router_fwd_var.cu -- the router forward with the router variants compiled in (sigmoid gate with a
+// selection bias, top-k-masked bin sums of eq. (12)); the kernels are in router_fwd_tc.cuh and
+// router_fwd_f32.cuh.
+#include "router_fwd_f32.cuh"
 
 namespace smoes {
 
@@ -9,6 +9,10 @@ cudaError_t launch_router_fwd_bf16_var(const FwdParams& p, const CUtensorMap& tm
                                        const CUtensorMap& tmW, const CUtensorMap* tmG, int n_sms,
                                        cudaStream_t s) {
   return launch_fwd_tc<true>(p, tmX, tmW, tmG, n_sms, s);
+}
+
+cudaError_t launch_router_fwd_f32_var(const FwdParams& p, cudaStream_t s) {
+  return launch_fwd_f32<true>(p, s);
 }
 
 }  // namespace smoes

@@ -297,6 +297,7 @@ cudaError_t launch_router_fwd_bf16_var(const FwdParams& p, const CUtensorMap& tm
                                        const CUtensorMap& tmW, const CUtensorMap* tmG, int n_sms,
                                        cudaStream_t s);   // router variants compiled in
 cudaError_t launch_router_fwd_f32(const FwdParams& p, cudaStream_t s);
+cudaError_t launch_router_fwd_f32_var(const FwdParams& p, cudaStream_t s);   // router variants compiled in
 int f32_chunks(int d);     // feature chunks of the fp32 forward and backward (128 features each)
 cudaError_t launch_router_bwd_bf16(const BwdParams& p, const CUtensorMap& tmX,
                                    const CUtensorMap& tmW, const CUtensorMap& tmDX,
