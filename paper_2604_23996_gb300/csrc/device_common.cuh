@@ -44,10 +44,11 @@ __device__ __forceinline__ float gauss_gc(const float* gcoef, int dcoef) {
   return -0.5f * t;
 }
 
+// 1 / (1 + e^-y) for y >= 0 and e^y / (1 + e^y) below: one exponential and one division for both (as
+// two branches a warp of mixed signs evaluated both).
 __device__ __forceinline__ float sigmoid_acc(float y) {
-  if (y >= 0.f) return 1.f / (1.f + expf(-y));
-  const float e = expf(y);
-  return e / (1.f + e);
+  const float e = expf(-fabsf(y));
+  return (y >= 0.f ? 1.f : e) / (1.f + e);
 }
 
 // Transpose-reduce of 32 values per lane: afterwards v[0] of lane l holds the sum over the 32

@@ -393,48 +393,8 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
   const uint32_t imask = (1u << (32 - __clz(max(nch * 16 - 1, 1)))) - 1u;
   const uint32_t xph = static_cast<uint32_t>(lt & 1);
 
-  // pass A: row maximum and top-k keys of this group's columns
-  constexpr int L = topk_len(KM);
-  float tk[L];
-#pragma unroll
-  for (int i = 0; i < L; ++i) tk[i] = -CUDART_INF_F;
-  float mx = -CUDART_INF_F, mx2 = -CUDART_INF_F;
-#pragma unroll 1
-  for (int c = cb; c < ce; ++c) {
-    float v[16];
-    src.load16(c, v);
-#pragma unroll
-    for (int t = 0; t < 16; t += 2) {
-      mx = fmaxf(mx, v[t]);
-      mx2 = fmaxf(mx2, v[t + 1]);
-    }
-    if (v_gate) {                    // sigmoid gate: the choice ranks s + bias (padding stays last)
-#pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        const int e = c * 16 + t;
-        v[t] = e < E ? sigmoid_acc(v[t]) + (p.score_bias ? __ldg(p.score_bias + e) : 0.f) : -FLT_MAX;
-      }
-    }
-    topk_take16<L>(tk, v, c, imask);
-  }
-  mx = fmaxf(mx, mx2);
-  es.xmax[grp * 128 + row] = mx;
-  if (grp == 1 && split) {
-#pragma unroll
-    for (int i = 0; i < L; ++i) es.xtk[i * 128 + row] = tk[i];
-  }
-  mbar_arrive(es.xbar + 0);
-  if (!mbar_wait(es.xbar + 0, xph, wc)) return;
-  mx = fmaxf(es.xmax[row], es.xmax[128 + row]);
-  if (grp == 0 && split) {
-    float o[L];
-#pragma unroll
-    for (int i = 0; i < L; ++i) o[i] = es.xtk[i * 128 + row];
-    topk_merge<L>(tk, o);
-  }
-
-  // pass B: e = exp(z - max), its sum, the bin sums of e and the saved scores
-  const float mxl = mx * kLog2e;
+  // what becomes of a 16-column chunk's gate values (saved exp(z - max), or s of the sigmoid gate):
+  // their sum, the saved scores and the bin sums
   float* grow = p.ws.gsave + static_cast<size_t>(valid ? j : 0) * E;
   float* prow = es.p_s + row;                       // p_s[b][row] at prow[b * kPsStride]
   const bool vec = (E & 3) == 0;
@@ -443,25 +403,10 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
   int cnt = 0, bin = split && grp ? 16 * nc0 / dm.N_B : 0;
   if (!dm.contig_bins && grp == 0)
     for (int b = 0; b < K; ++b) prow[b * kPsStride] = 0.f;
-  if (stg && lt > 0 && !mbar_wait(es.stg_free + grp, static_cast<uint32_t>((lt - 1) & 1), wc)) return;
-#pragma unroll 1
-  for (int c = cb; c < ce; ++c) {
-    float v[16];
-    src.load16(c, v);
+  auto emit = [&](int c, const float (&v)[16]) {
     float ps[4] = {0.f, 0.f, 0.f, 0.f};
-    if (!v_gate) {
 #pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        v[t] = exp2f(fmaf(v[t], kLog2e, -mxl));                 // saved e = exp(z - max)
-        ps[t & 3] += v[t];
-      }
-    } else {
-#pragma unroll
-      for (int t = 0; t < 16; ++t) {
-        v[t] = sigmoid_acc(v[t]);                               // saved s = sigmoid(z)
-        ps[t & 3] += v[t];
-      }
-    }
+    for (int t = 0; t < 16; ++t) ps[t & 3] += v[t];
     sum += (ps[0] + ps[1]) + (ps[2] + ps[3]);
     if (stg) {
       uint8_t* rb = es.stg + (c >> 1) * 16384 + row * 128;
@@ -499,6 +444,65 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
 #pragma unroll
       for (int t = 0; t < 16; ++t)
         if (c * 16 + t < E) prow[__ldg(p.ws.expert_bin + c * 16 + t) * kPsStride] += v[t];
+    }
+  };
+
+  // pass A: row maximum and top-k keys of this group's columns. The sigmoid gate needs no maximum: its
+  // values are formed once and emitted here.
+  constexpr int L = topk_len(KM);
+  float tk[L];
+#pragma unroll
+  for (int i = 0; i < L; ++i) tk[i] = -CUDART_INF_F;
+  float mx = -CUDART_INF_F, mx2 = -CUDART_INF_F;
+  if (v_gate && stg && lt > 0 && !mbar_wait(es.stg_free + grp, static_cast<uint32_t>((lt - 1) & 1), wc)) return;
+#pragma unroll 1
+  for (int c = cb; c < ce; ++c) {
+    float v[16];
+    src.load16(c, v);
+#pragma unroll
+    for (int t = 0; t < 16; t += 2) {
+      mx = fmaxf(mx, v[t]);
+      mx2 = fmaxf(mx2, v[t + 1]);
+    }
+    if (v_gate) {                    // the choice ranks s + bias (padding stays last)
+#pragma unroll
+      for (int t = 0; t < 16; ++t) v[t] = sigmoid_acc(v[t]);
+      emit(c, v);
+#pragma unroll
+      for (int t = 0; t < 16; ++t) {
+        const int e = c * 16 + t;
+        v[t] = e < E ? v[t] + (p.score_bias ? __ldg(p.score_bias + e) : 0.f) : -FLT_MAX;
+      }
+    }
+    topk_take16<L>(tk, v, c, imask);
+  }
+  mx = fmaxf(mx, mx2);
+  es.xmax[grp * 128 + row] = mx;
+  if (grp == 1 && split) {
+#pragma unroll
+    for (int i = 0; i < L; ++i) es.xtk[i * 128 + row] = tk[i];
+  }
+  mbar_arrive(es.xbar + 0);
+  if (!mbar_wait(es.xbar + 0, xph, wc)) return;
+  mx = fmaxf(es.xmax[row], es.xmax[128 + row]);
+  if (grp == 0 && split) {
+    float o[L];
+#pragma unroll
+    for (int i = 0; i < L; ++i) o[i] = es.xtk[i * 128 + row];
+    topk_merge<L>(tk, o);
+  }
+
+  // pass B: e = exp(z - max), its sum, the bin sums of e and the saved scores
+  const float mxl = mx * kLog2e;
+  if (!v_gate) {
+    if (stg && lt > 0 && !mbar_wait(es.stg_free + grp, static_cast<uint32_t>((lt - 1) & 1), wc)) return;
+#pragma unroll 1
+    for (int c = cb; c < ce; ++c) {
+      float v[16];
+      src.load16(c, v);
+#pragma unroll
+      for (int t = 0; t < 16; ++t) v[t] = exp2f(fmaf(v[t], kLog2e, -mxl));   // saved e = exp(z - max)
+      emit(c, v);
     }
   }
   release();
@@ -1282,7 +1286,8 @@ cudaError_t launch_fwd_tc(const FwdParams& p, const CUtensorMap& tmX, const CUte
     while (n > 2 && fwd_smem_bytes(N, n, p.dm.d, p.dm.K, p.dm.E, gauss, stg) > 227u * 1024u) --n;
     return n;
   };
-  const bool one_tile = p.n_tiles <= n_sms &&
+  // (the sigmoid gate stages in pass A, before that exchange)
+  const bool one_tile = p.n_tiles <= n_sms && !p.dm.gate &&
                         stages_for(false) * fwd_stage_bytes(N) >= kPermScratchBytes + fwd_stg_bytes(p.dm.E);
   const int use_stg = tmG == nullptr ? kStgNone : one_tile ? kStgInRing : stages_for(true) >= 5 ? kStgOwn : kStgNone;
   const int n_stages = stages_for(use_stg == kStgOwn);
