@@ -195,7 +195,7 @@ k_router_fwd_f32(const FwdParams p) {
     const EpiSmem es = epi_smem(epi, dm.K, bars);
     uint32_t n_in = 0;
     const TileMeta meta = load_tile_meta(p, tile, row);   // (no fused permutation on this path)
-    epilogue_tile<KM, kVar>(p, src, rel, tile, grp, row, 0, kGauss ? dll_s[row] : 0.f, meta, es, wc, n_in, true);
+    epilogue_tile<KM, kVar, false>(p, src, rel, tile, grp, row, 0, kGauss ? dll_s[row] : 0.f, meta, es, wc, n_in, true);
   }
 }
 

@@ -98,6 +98,13 @@ __device__ __forceinline__ void topk_merge(float (&tk)[L], const float (&v)[L]) 
       if ((i & j) == 0) cmp_desc(tk[i], tk[i + j]);
   }
 }
+// 2^x on the special-function unit: exp2f's value, without its scaling of results below 2^-126.
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // The keys of 16 logits (experts 16 c + t) into the running list.
 template <int L>
 __device__ __forceinline__ void topk_take16(float (&tk)[L], const float (&v)[16], int c, uint32_t imask) {
@@ -306,6 +313,7 @@ struct EpiSmem {
   float* xtk;            // [kMaxTopK][128] group 1's top-k keys of each row
   uint64_t* bar_in;      // count 256: the partials of one (tile, sample) are written
   uint64_t* bar_out;     // count 256: the tile's pieces are written
+  uint64_t* bar_red;     // count 1: the reducer warp is done with the tile
   uint64_t* xbar;        // [3] count 256: row maxima and keys / row sums / row tables exchanged
   uint64_t* perm_go;     // count 1: the CTA's top-k and pair counts are complete
   // optional staging of the tile's scores for coalesced TMA stores: 32-column blocks of
@@ -338,6 +346,7 @@ __device__ inline EpiSmem epi_smem(float* base, int K, uint64_t* bars) {
   es.bar_out = bars + 1;
   es.xbar = bars + 2;
   es.perm_go = nullptr;
+  es.bar_red = nullptr;
   es.stg = nullptr;
   es.stg_full = es.stg_free = nullptr;
   es.tmG = nullptr;
@@ -360,12 +369,35 @@ __device__ __forceinline__ int epi_split(const Dims& dm) {
   return nc0;
 }
 
+// Announces a tile's pieces (complete, and ordered by a fence before) and reduces the samples that
+// they complete; run by one warp.
+__device__ __forceinline__ void announce_pieces(const FwdParams& p, const TileMeta& meta, float* red) {
+  const int lane = threadIdx.x & 31;
+  const int s0 = meta.s0, s1 = meta.s1;
+  for (int s = s0; s <= s1; ++s) {
+    // a sample strictly inside the tile has this tile's piece only
+    const int pb = s == s0 ? meta.pb0 : s == s1 ? meta.pb1 : meta.pbase + (s - s0);
+    const int pe = s == s0 ? meta.pe0 : s == s1 ? meta.pe1 : pb + 1;
+    const int nt = s == s0 ? meta.n0 : s == s1 ? meta.n1 : 0;
+    uint32_t last = 0;
+    if (lane == 0) last = (atomicAdd(p.ws.sample_ticket + s, 1u) + 1u == static_cast<uint32_t>(pe - pb));
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (last) {
+      __threadfence();
+      const bool known = s == s0 || s == s1;
+      sample_reduce(p, s, red, known ? pb : -1, pe, nt, false);
+    }
+  }
+}
+
 // Per-tile epilogue, run by both groups (grp 0, 1) for every tile. Src::load16(c, v) returns
 // logits [16c, 16c+16) of this thread's row, -FLT_MAX past E (finite, so that its top-k key is
 // not a NaN; warp-collective); release() is called after the last logit read. row: token row in
 // the tile (0..127); lt: index of the tile among those this CTA processes; dll: the row's
 // Gaussian log-likelihood difference (read by group 1); meta: the tile's metadata
-// (load_tile_meta); n_in: completed phases of bar_in (identical in all 256 threads).
+// (load_tile_meta); n_in: completed phases of bar_in (identical in all 256 threads). kReducer: a warp
+// of its own announces the pieces and reduces samples (the fence alone held all eight warps for 2 us
+// of a 128-expert tile's 15); otherwise the first warp does.
 //
 // Softmax in two passes over each group's columns: pass A finds the row maximum and top-k keys
 // (merged across the groups through shared memory); pass B forms e = exp(z - max), its row sum,
@@ -375,7 +407,7 @@ __device__ __forceinline__ int epi_split(const Dims& dm) {
 // joint table (eq. 12), each a half of the values. With the fused permutation, the first thread
 // arrives on es.perm_go as soon as the rows of the CTA's last tile are counted (the partial sums
 // and their fence follow).
-template <int KM, bool kVar, class Src, class Release>
+template <int KM, bool kVar, bool kReducer, class Src, class Release>
 __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release& release, int tile,
                               int grp, int row, int lt, float dll, const TileMeta& meta,
                               const EpiSmem& es, const WaitCtx& wc, uint32_t& n_in, bool last_tile) {
@@ -501,7 +533,7 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
       float v[16];
       src.load16(c, v);
 #pragma unroll
-      for (int t = 0; t < 16; ++t) v[t] = exp2f(fmaf(v[t], kLog2e, -mxl));   // saved e = exp(z - max)
+      for (int t = 0; t < 16; ++t) v[t] = ex2_ftz(fmaf(v[t], kLog2e, -mxl));   // saved e = exp(z - max)
       emit(c, v);
     }
   }
@@ -674,27 +706,15 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
     tma_store_wait_read<0>();
     mbar_arrive(es.stg_free + grp);
   }
-  __threadfence();
+  if (!kReducer) __threadfence();
+  // (the reducer warp, a tile behind at most, orders the pieces with its own fence)
+  if (kReducer && lt > 0 && !mbar_wait(es.bar_red, static_cast<uint32_t>((lt - 1) & 1), wc)) return;
   mbar_arrive(es.bar_out);
-  if (grp == 0 && wg == 0) {            // the first warp announces the pieces, reduces samples
+  if (!kReducer && grp == 0 && wg == 0) {
     bool ok = true;
     if (lane == 0) ok = mbar_wait(es.bar_out, static_cast<uint32_t>(lt & 1), wc);
     ok = __shfl_sync(0xffffffffu, ok, 0);
-    if (!ok) return;
-    for (int s = s0; s <= s1; ++s) {
-      // a sample strictly inside the tile has this tile's piece only
-      const int pb = s == s0 ? meta.pb0 : s == s1 ? meta.pb1 : meta.pbase + (s - s0);
-      const int pe = s == s0 ? meta.pe0 : s == s1 ? meta.pe1 : pb + 1;
-      const int nt = s == s0 ? meta.n0 : s == s1 ? meta.n1 : 0;
-      uint32_t last = 0;
-      if (lane == 0) last = (atomicAdd(p.ws.sample_ticket + s, 1u) + 1u == static_cast<uint32_t>(pe - pb));
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (last) {
-        __threadfence();
-        const bool known = s == s0 || s == s1;
-        sample_reduce(p, s, es.red, known ? pb : -1, pe, nt, false);
-      }
-    }
+    if (ok) announce_pieces(p, meta, es.red);
   }
 }
 
@@ -895,15 +915,16 @@ __host__ __device__ inline size_t fwd_smem_bytes(int N, int n_stages, int d, int
   if (stg) b += fwd_stg_bytes(E);
   if (gauss) b += 2u * sizeof(float) * static_cast<size_t>(round_up(d, kFwdBK));
   b += sizeof(float) * (epi_smem_floats(K) + 256u + 8u);
-  b += sizeof(uint64_t) * (2u * n_stages + 19u + kEpiBars + kCoefBars);
+  b += sizeof(uint64_t) * (2u * n_stages + 20u + kEpiBars + kCoefBars);
   b += 16u;
   return b + 1024u;   // alignment slack
 }
 
 // Roles: warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue group 0, then (Gaussian
 // score) warps 6-9 Gaussian and 10-13 epilogue group 1, or (provided scores) warps 6-9 epilogue
-// group 1. With 14 warps four share a sub-partition's 16K registers: 128 per thread.
-constexpr int fwd_threads(bool gauss) { return gauss ? 448 : 320; }
+// group 1; the last warp reduces samples. With 15 warps four share a sub-partition's 16K registers:
+// 128 per thread.
+constexpr int fwd_threads(bool gauss) { return gauss ? 480 : 352; }
 
 template <bool kGauss, int KM, bool kVar>
 __global__ void __launch_bounds__(fwd_threads(kGauss), 1)
@@ -947,6 +968,7 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint64_t* perm_go = reinterpret_cast<uint64_t*>(q);   q += 8;
   uint64_t* stg_full = reinterpret_cast<uint64_t*>(q);  q += 16;
   uint64_t* stg_free = reinterpret_cast<uint64_t*>(q);  q += 16;
+  uint64_t* bar_red = reinterpret_cast<uint64_t*>(q);   q += 8;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q); q += 4;
   int* abort_flag = reinterpret_cast<int*>(q);
 
@@ -974,6 +996,7 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     mbar_init(coef_issued, 256);
     mbar_init(gc_bar, 256);
     mbar_init(perm_go, 1);
+    mbar_init(bar_red, 1);
     int* ctot = epi_smem(epi, dm.K, ebars).ctot;
     for (int i = 0; i < kMaxBins; ++i) ctot[i] = 0;
     fence_mbar_init();
@@ -1126,6 +1149,20 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     int dummy = 0;
     wd.abort_flag = &dummy;
     mbar_wait(drain, 0, wd);
+  } else if (warp == (kGauss ? 14 : 10)) {
+    // ---------------------------------------------------------------- sample reducer
+    const EpiSmem es = epi_smem(epi, dm.K, ebars);
+    // the sample reduction's code into the instruction cache while the first tile streams in
+    sample_reduce(p, 0, es.red, 0, 1, 1, true);
+    int lt = 0;
+    for (int tile = t_beg; tile < t_end; ++tile, ++lt) {
+      const TileMeta meta = load_tile_meta(p, tile, lane);   // lands while the tile streams in
+      if (!warp_wait(es.bar_out, static_cast<uint32_t>(lt & 1), wc)) break;
+      __threadfence();                       // the pieces of all 256 threads, before the tickets
+      announce_pieces(p, meta, es.red);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_red);
+    }
   } else if (warp < 6 || warp >= (kGauss ? 10 : 6)) {
     // ---------------------------------------------------------------- epilogue (2 x 4 warps)
     const int grp = warp < 6 ? 0 : 1;        // column half of the logits
@@ -1133,6 +1170,7 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     const int row = lg * 32 + lane;          // tile row == TMEM lane == token offset
     EpiSmem es = epi_smem(epi, dm.K, ebars);
     es.perm_go = perm_go;
+    es.bar_red = bar_red;
     if (use_stg) {
       es.stg = stg;
       es.stg_full = stg_full;
@@ -1161,8 +1199,6 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       for (int w = 0; w < 8; ++w) gc += gred[w];
       gc *= -0.5f;
     }
-    // the sample reduction's code into the instruction cache while the first tile streams in
-    if (grp == 0 && lg == 0) sample_reduce(p, 0, es.red, 0, 1, 1, true);
     uint32_t n_in = 0;
     int lt = 0;
     for (int tile = t_beg; tile < t_end; ++tile, ++lt) {
@@ -1177,7 +1213,7 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         dll = dll_s[buf * 128 + row] + gc;
         mbar_arrive(g_empty + buf);
       }
-      epilogue_tile<KM, kVar>(p, Src{tl + static_cast<uint32_t>(buf * N), dm.E}, Rel{acc_empty + buf},
+      epilogue_tile<KM, kVar, true>(p, Src{tl + static_cast<uint32_t>(buf * N), dm.E}, Rel{acc_empty + buf},
                         tile, grp, row, lt, dll, meta, es, wc, n_in, tile == t_end - 1);
     }
     if (use_stg && row == 0) tma_store_wait_all<0>();   // the score stores complete before exit
