@@ -690,6 +690,7 @@ smoes_status smoes_router_bwd(smoes_plan P, const void* X, const void* W, const 
   p.n_tiles = P->bwd_tiles;
   p.limit_ns = P->limit_ns;
   p.balance_armed = P->balance_armed ? 1 : 0;
+  p.n_sms = P->n_sms;
   cudaError_t e;
   if (d.dtype == SMOES_BF16) {
     const int E_pad = round_up(d.E, 64);

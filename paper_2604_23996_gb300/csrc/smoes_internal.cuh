@@ -129,6 +129,7 @@ struct BwdParams {
   int n_tiles;               // token tiles
   uint64_t limit_ns;
   int balance_armed;         // host's view: smoes_bin_balance was called since the last forward
+  int n_sms;
 };
 
 struct PermParams {
