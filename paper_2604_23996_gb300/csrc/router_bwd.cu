@@ -371,10 +371,10 @@ constexpr int kDxBufs = 4;
 constexpr int kDrainGroups = 2;
 constexpr int kBwdThreads = 64 + kDrainGroups * 128;
 
-__host__ __device__ inline BwdLayout bwd_layout(int E_pad, int n_xst) {
+__host__ __device__ inline BwdLayout bwd_layout(int E_pad, int slice_width, int n_xst) {
   BwdLayout L;
   uint32_t o = 0;
-  L.wsl = o;  o += 65536u;                                         // W slice (ds * E_pad * 2 B)
+  L.wsl = o;  o += static_cast<uint32_t>(slice_width * E_pad) * 2u;   // W slice, 128 columns per d-block
   L.dz = o;   o += 2u * 2u * static_cast<uint32_t>(E_pad) * 128u;   // 2 buffers x (hi, lo)
   L.xst = o;  o += static_cast<uint32_t>(n_xst) * 16384u;          // X stages [2 atoms][64][128 B]
   L.stg = o;  o += kDrainGroups * 16384u;                          // dX staging [2 atoms][64][128 B] per group
@@ -396,7 +396,7 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const Dims& dm = p.dm;
-  const BwdLayout L = bwd_layout(E_pad, n_xst);
+  const BwdLayout L = bwd_layout(E_pad, p.slice_width, n_xst);
   uint8_t* wsl = base + L.wsl;
   uint8_t* dzb = base + L.dz;               // buffer zb: hi at zb*2*E_pad*128, lo right after
   uint8_t* xst = base + L.xst;
@@ -882,8 +882,8 @@ cudaError_t launch_router_bwd_bf16(const BwdParams& p, const CUtensorMap& tmX, c
   const int E_pad = round_up(p.dm.E, 64);
   if (E_pad > 128) return cudaErrorInvalidValue;
   int n_xst = 6;
-  while (n_xst > 2 && bwd_layout(E_pad, n_xst).total > 227u * 1024u) --n_xst;
-  const uint32_t smem = bwd_layout(E_pad, n_xst).total;
+  while (n_xst > 2 && bwd_layout(E_pad, p.slice_width, n_xst).total > 227u * 1024u) --n_xst;
+  const uint32_t smem = bwd_layout(E_pad, p.slice_width, n_xst).total;
   if (smem > 227u * 1024u) return cudaErrorInvalidConfiguration;
   auto k = (E_pad == 64) ? k_router_bwd_tc<64> : k_router_bwd_tc<128>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
