@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kFinSlices * kFinCols) k_stats_finalize(const 
   const int i = i2 < 2 * p.d ? i2 % p.d : 0;
   const int G = p.G;
   const size_t at = static_cast<size_t>(m) * p.d + i;
-  double N0 = 0.0, Smu0 = 0.0, Svar0 = 0.0;
+  double N0 = 0.0, Smu0 = 0.0, Svar0 = 0.0, inv_N0 = 0.0, mean0 = 0.0;
   if (sl == 0) {
     N0 = p.N0[m];
     Smu0 = p.S_mu[at];
@@ -299,8 +299,10 @@ __global__ void __launch_bounds__(kFinSlices * kFinCols) k_stats_finalize(const 
     if (col < 2) inv_n_s[col] = cnt > 0 ? 1.0 / cnt : 0.0;
     if (col == 0) cnt_s = nvis;
   }
-  const double inv_N0 = 1.0 / N0;
-  const double mean0 = div_by(Smu0, N0, inv_N0);  // S_mu,t-1 / N_t-1 (used when N0 > 0)
+  if (sl == 0) {                                  // (one warp of the block: fp64 is scarce)
+    inv_N0 = 1.0 / N0;
+    mean0 = div_by(Smu0, N0, inv_N0);             // S_mu,t-1 / N_t-1 (used when N0 > 0)
+  }
   red[0][sl][col] = a1;
   red[1][sl][col] = a2;
   __syncthreads();
