@@ -43,13 +43,19 @@ __device__ __forceinline__ void empty_sel(TokenSel<KM>& s) {
   s.m = 0;
 }
 
+// Token j's top-k and modality from memory, and the selection they make.
 template <int KM>
-__device__ __forceinline__ void load_sel(const PermParams& p, const uint8_t* s_pos, int j, TokenSel<KM>& s) {
-  empty_sel<KM>(s);
-  int e[KM];
+__device__ __forceinline__ void load_topk(const PermParams& p, int j, int (&e)[KM], int& m) {
+  m = 0;
 #pragma unroll
-  for (int i = 0; i < KM; ++i) e[i] = i < p.k ? p.topk_idx[static_cast<size_t>(j) * p.k + i] : -1;
-  s.m = (p.is_vision && !p.is_vision[j]) ? 1 : 0;
+  for (int i = 0; i < KM; ++i) e[i] = (j < p.T && i < p.k) ? __ldg(p.topk_idx + static_cast<size_t>(j) * p.k + i) : -1;
+  if (j < p.T && p.is_vision) m = __ldg(p.is_vision + j) ? 0 : 1;
+}
+template <int KM>
+__device__ __forceinline__ void make_sel(const PermParams& p, const uint8_t* s_pos, const int (&e)[KM], int m,
+                                         TokenSel<KM>& s) {
+  empty_sel<KM>(s);
+  s.m = m;
 #pragma unroll
   for (int i = 0; i < KM; ++i) {
     if (i < p.k) {
@@ -90,6 +96,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int K = p.K, NB = p.E / p.K;
   const uint32_t nb_mask = NB >= 32 ? 0xffffffffu : (1u << NB) - 1u;
+  int e0[KM], m0;                                       // the first round's top-k, beside the tables
+  load_topk<KM>(p, blockIdx.x * p.rounds * kPermThreads + threadIdx.x, e0, m0);
   for (int e = threadIdx.x; e < p.E; e += kPermThreads) s_pos[e] = static_cast<uint8_t>(p.expert_bin[e] * NB + p.expert_slot[e]);
   for (int i = threadIdx.x; i < K * K; i += kPermThreads) disp[i] = 0;
   for (int i = threadIdx.x; i < 2 * p.E; i += kPermThreads) ecnt[i] = 0;
@@ -104,7 +112,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
     const int j = (blockIdx.x * p.rounds + r) * kPermThreads + threadIdx.x;
     TokenSel<KM> s;
     empty_sel<KM>(s);
-    if (j < p.T) load_sel<KM>(p, s_pos, j, s);
+    if (r > 0) load_topk<KM>(p, j, e0, m0);
+    if (j < p.T) make_sel<KM>(p, s_pos, e0, m0, s);
     if (r == 0) s0 = s;
     for (int kb = 0; kb < K; ++kb) {
       const int c = __popc(__ballot_sync(0xffffffffu, next_mask(s.set, NB, nb_mask) != 0u));
@@ -191,7 +200,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm(const PermParams p) {
       s = s0;
     } else {
       empty_sel<KM>(s);
-      if (valid) load_sel<KM>(p, s_pos, j, s);
+      load_topk<KM>(p, j, e0, m0);
+      if (valid) make_sel<KM>(p, s_pos, e0, m0, s);
     }
     if (p.rounds > 1) {                                 // (one round: wcnt still holds the warps' counts)
       uint32_t set[kSetWords];
