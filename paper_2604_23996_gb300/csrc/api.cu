@@ -386,7 +386,7 @@ smoes_status smoes_plan_create(const smoes_router_desc* desc, smoes_plan* out) {
   L.attn_part = take(sizeof(float) * static_cast<size_t>(T) * std::max(0, d.attn_max_heads));
   L.gcoef = take(sizeof(float) * (2 * static_cast<size_t>(P->dcoef) + P->dcoef / 256));
   P->stat_blocks = stats_blocks(T, P->n_sms);
-  P->bal_blocks = std::max(1, std::min(2 * P->n_sms, (T + 63) / 64));
+  P->bal_blocks = std::max(1, std::min(2 * P->n_sms, (T + 31) / 32));   // (one round of loads per warp up to 9728 tokens)
   L.stat_part = take(sizeof(float) * 4 * static_cast<size_t>(P->stat_blocks) * d.d);
   L.stat_nvis = take(sizeof(int32_t) * static_cast<size_t>(P->stat_blocks));
   L.stat_n0 = take(sizeof(double) * 2);
@@ -814,6 +814,7 @@ smoes_status smoes_bin_balance(smoes_plan P, const int32_t* topk_idx, float loss
   p.gsave = v.gsave;
   p.topk_idx = topk_idx;
   p.expert_bin = v.expert_bin;
+  p.expert_slot = v.expert_slot;
   p.expert_bin_host = P->expert_bin.data();
   p.scale = loss_scale;
   p.part_h = reinterpret_cast<float*>(b + P->L.bal_h);

@@ -218,7 +218,8 @@ __global__ void __launch_bounds__(kBalThreads) k_bal_partial_pow2(const BalParam
 // One block of 1024 threads (plans hold E <= 128), all in fp32 and integers. The block partials
 // of each expert are summed in eight slices of the blocks, each slice with its loads issued
 // together and added in block order, then the slices in slice order; the per-bin token counts the
-// same way in integers. Every later step runs one thread per expert or per bin. (The sums are
+// same way in integers. Every later step runs one thread per expert or per bin; a bin's thread walks
+// its own N_B experts by slot (a search through all of them was most of this kernel's time). (The sums are
 // fixed-order and so bitwise reproducible; fp64 is avoided because on GB300 each fp64 operation
 // in these short dependent chains costs far more than the fp32 one, and the fp32 rounding of
 // sums over a few hundred partials is far inside the 2e-3 tolerance of the outputs.)
@@ -233,13 +234,17 @@ __global__ void __launch_bounds__(kFinThreads) k_bal_finalize(const BalParams p)
   __shared__ int u_sl[kFinSl][kMaxBins];
   __shared__ float f_s[kFinRow], P_s[kFinRow], H_s[kFinRow], term_s[kMaxBins];
   __shared__ int sel_s[kFinRow], bin_sel[kMaxBins], bin_u[kMaxBins];
-  __shared__ int eb_s[kFinRow];
+  __shared__ int eb_s[kFinRow], exp_s[kFinRow];     // bin of an expert; expert at bin * N_B + slot
   pdl_wait();                                       // the block partials
   pdl_trigger();
   const int E = p.E, K = p.K, G = p.G;
   const int tid = threadIdx.x;
   const int e = tid % kFinRow, sl = tid / kFinRow;
-  if (tid < E) eb_s[tid] = __ldg(p.expert_bin + tid);
+  if (tid < E) {
+    const int kb = __ldg(p.expert_bin + tid);
+    eb_s[tid] = kb;
+    exp_s[kb * p.N_B + __ldg(p.expert_slot + tid)] = tid;
+  }
   {
     const int g0 = sl * G / kFinSl, g1 = (sl + 1) * G / kFinSl;
     float H = 0.f;
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(kFinThreads) k_bal_finalize(const BalParams p)
   __syncthreads();
   if (tid < K) {                                    // selections of each bin's experts (counts < 2^24)
     int t = 0;
-    for (int x = 0; x < E; ++x) t += eb_s[x] == tid ? sel_s[x] : 0;
+    for (int i = 0; i < p.N_B; ++i) t += sel_s[exp_s[tid * p.N_B + i]];
     bin_sel[tid] = t;
   }
   __syncthreads();
@@ -304,8 +309,10 @@ __global__ void __launch_bounds__(kFinThreads) k_bal_finalize(const BalParams p)
   __syncthreads();
   if (tid < K) {                                    // eq. (16): bin tid's term, its experts in order
     float t = 0.f;
-    for (int x = 0; x < E; ++x)
-      if (eb_s[x] == tid) t = fmaf(f_s[x], P_s[x], t);
+    for (int i = 0; i < p.N_B; ++i) {
+      const int x = exp_s[tid * p.N_B + i];
+      t = fmaf(f_s[x], P_s[x], t);
+    }
     term_s[tid] = NB * t;
   }
   __syncthreads();
