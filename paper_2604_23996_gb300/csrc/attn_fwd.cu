@@ -79,16 +79,17 @@ struct AttnItem {
   int b, h, qt0, nq;          // first query tile, tiles in the pair (1 or 2)
 };
 
+template <int kTiles>       // query tiles per item: 2, or 1 (see the launch)
 __device__ __forceinline__ AttnItem decode_item(const AttnParams& p, int item) {
-  const int n_pairs = (p.n_qtiles + 1) / 2;
+  const int n_pairs = (p.n_qtiles + kTiles - 1) / kTiles;
   const int BH = p.B * p.H;
   const int pr = n_pairs - 1 - item / BH;
   const int bh = item - (item / BH) * BH;
   AttnItem it;
   it.b = bh / p.H;
   it.h = bh - it.b * p.H;
-  it.qt0 = 2 * pr;
-  it.nq = min(2, p.n_qtiles - it.qt0);
+  it.qt0 = kTiles * pr;
+  it.nq = min(kTiles, p.n_qtiles - it.qt0);
   return it;
 }
 
@@ -181,7 +182,7 @@ constexpr int kKtFloats = 2 * kKtKeys + kKtKeys / 32 * 4;   // bias * log2 e | c
 
 // The warp that stages (bias * log2 e, carried score) of the keys, four blocks at a time, keys past
 // S masked; loaded a stage ahead. kt: the stages, [kKtStages][kKtFloats]; full has count 32.
-template <bool kFloatM>
+template <bool kFloatM, int kTiles>
 __device__ __forceinline__ void stage_key_terms(const AttnParams& p, int n_items, float* kt, uint64_t* kt_full,
                                                 uint64_t* kt_empty, const WaitCtx& wc) {
   constexpr int kN = kKtKeys / 32;
@@ -192,7 +193,7 @@ __device__ __forceinline__ void stage_key_terms(const AttnParams& p, int n_items
   for (int rd = 0; ok; ++rd) {
     const int item = dealt_item(rd);
     if (item >= n_items) break;
-    const AttnItem w = decode_item(p, item);
+    const AttnItem w = decode_item<kTiles>(p, item);
     const int nkb = kblocks_of(p, w.qt0 + w.nq - 1);
     for (int kb = 0; kb < nkb; kb += kKtBlocks) {
       float b[kN], m[kN];
@@ -355,7 +356,7 @@ __host__ __device__ inline AttnLayout attn_layout() {
   return L;
 }
 
-template <bool kFloatM>
+template <bool kFloatM, int kTiles>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const AttnFwdParams fp) {
@@ -389,7 +390,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   float* mrg = reinterpret_cast<float*>(base + L.mrg);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int n_items = ((p.n_qtiles + 1) / 2) * p.B * p.H;
+  const int n_items = ((p.n_qtiles + kTiles - 1) / kTiles) * p.B * p.H;
   WaitCtx wc{abort_flag, p.status, p.limit_ns};
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -439,7 +440,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       for (int rd = 0; ok; ++rd) {
         const int item = dealt_item(rd);
         if (item >= n_items) break;
-        const AttnItem w = decode_item(p, item);
+        const AttnItem w = decode_item<kTiles>(p, item);
         const int row0 = (w.b * p.H + w.h) * p.S, krow0 = (w.b * fp.Hkv + w.h / G) * p.S;
         for (int t = 0; t < w.nq && ok; ++t) {
           if (!warp_wait(q_empty + t, (static_cast<uint32_t>(nqt[t]) & 1u) ^ 1u, wc)) { ok = false; break; }
@@ -499,7 +500,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       for (int rd = 0; ok; ++rd) {
         const int item = dealt_item(rd);
         if (item >= n_items) break;
-        const AttnItem w = decode_item(p, item);
+        const AttnItem w = decode_item<kTiles>(p, item);
         int nb[2];
         nb[0] = kblocks_of(p, w.qt0);
         nb[1] = w.nq > 1 ? kblocks_of(p, w.qt0 + 1) : 0;
@@ -569,7 +570,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       mbar_wait(drain, 0, wd);
     }
   } else if (warp == 2) {
-    stage_key_terms<kFloatM>(p, n_items, kt, kt_full, kt_empty, wc);
+    stage_key_terms<kFloatM, kTiles>(p, n_items, kt, kt_full, kt_empty, wc);
   } else if (warp >= 4) {
     // ---------------------------------------------------------------- softmax groups (4 x 4 warps)
     attn_more_registers();
@@ -590,7 +591,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     for (int rd = 0; ok; ++rd) {
       const int item = dealt_item(rd);
       if (item >= n_items) break;
-      const AttnItem w = decode_item(p, item);
+      const AttnItem w = decode_item<kTiles>(p, item);
       const int qt = w.qt0 + t;
       const int nkb = kblocks_of(p, w.qt0 + w.nq - 1);
       const int mine = t < w.nq ? kblocks_of(p, qt) : 0;
@@ -724,9 +725,14 @@ cudaError_t launch_attn_fwd(const AttnFwdParams& fp, const CUtensorMap& tmQ, con
   const AttnParams& p = fp.a;
   if (p.hd != kAttnHd || p.S % kAttnTile != 0 || fp.Hkv < 1 || p.H % fp.Hkv != 0) return cudaErrorNotSupported;
   const uint32_t smem = attn_layout().total;
-  const int n_items = ((p.n_qtiles + 1) / 2) * p.B * p.H;
+  // one tile per item while every tile has an SM to itself: a pair's blocks take longer than one
+  // tile's (1 x 16 x 512: 20.1 against 16.6 us)
+  const int tiles = p.n_qtiles * p.B * p.H;
+  const bool single = tiles <= n_sms;
+  const int n_items = single ? tiles : ((p.n_qtiles + 1) / 2) * p.B * p.H;
   const int grid = n_items < n_sms ? n_items : n_sms;
-  auto k = p.m_prev ? k_attn_fwd<true> : k_attn_fwd<false>;
+  auto k = p.m_prev ? (single ? k_attn_fwd<true, 1> : k_attn_fwd<true, 2>)
+                    : (single ? k_attn_fwd<false, 1> : k_attn_fwd<false, 2>);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3(grid), dim3(kAttnThreads), smem, s, tmQ, tmK, tmV, fp);
