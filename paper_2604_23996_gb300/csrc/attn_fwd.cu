@@ -16,7 +16,7 @@
 // hide each other's softmax: with the weights in tensor memory nothing but Q, K and V needs
 // shared memory, and S, P and O of two tiles fill the 512 columns. One tile per CTA, its weights
 // in shared memory, had every step of a block wait for the one before: 8 x 16 x 4096 causal with
-// H_kv = 4 took 1270 us, now 607 us. Groups of a whole row (128 keys per thread, half the warps)
+// H_kv = 4 took 1270 us, now 556 us (607 us before the converged issue). Groups of a whole row (128 keys per thread, half the warps)
 // took 735 us with the scores in registers and 643 us reading them twice.
 #include <cuda_bf16.h>
 #include <math_constants.h>

@@ -12,12 +12,6 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Coefficients of one feature of the Gaussian log-likelihood difference of eq. (8),
 //   dLL(x) = LL_v - LL_t = sum_d ga[d] x_d^2 + gb[d] x_d + gc,
 //   ga = (var_v - var_t) / (2 var_v var_t),  gb = (mu_v var_t - mu_t var_v) / (var_v var_t),

@@ -366,7 +366,7 @@ struct BwdLayout {
 };
 
 // dX^T accumulators in TMEM: kDxBufs buffers of 64 columns after the dW^T blocks (which take at
-// most 256 columns: slice width x E_pad = 32768), drained by two warp groups in turn.
+// most 256 columns: two 128-column d-blocks of at most 128 experts), drained by two warp groups in turn.
 constexpr int kDxBufs = 4;
 constexpr int kDrainGroups = 2;
 constexpr int kBwdThreads = 64 + kDrainGroups * 128;

@@ -3,8 +3,8 @@
 // One pass over X computes, per token: the gate logits z = W x (Sec. 3.1) on tcgen05 tensor
 // cores (TMA-fed, accumulators in TMEM), the Gaussian modality score of eqs. (8)-(9) from the
 // same shared-memory X tiles, softmax, top-k, bin sums p_k = sum_{e in B_k} g_e, and the
-// per-(128-token tile, sample) partial sums of the joint table of eq. (12). The epilogue group
-// that completes the last partial of a sample reduces that sample's joint to P (eq. 13),
+// per-(128-token tile, sample) partial sums of the joint table of eq. (12). The reducer warp of the
+// CTA that completes the last partial of a sample reduces that sample's joint to P (eq. 13),
 // I (eq. 14) and the backward coefficient table; the one that completes the last sample writes
 // the loss of eq. (15). All reductions run in a fixed order: results are bitwise reproducible.
 //

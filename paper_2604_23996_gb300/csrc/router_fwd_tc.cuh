@@ -4,8 +4,8 @@
 // One pass over X computes, per token: the gate logits z = W x (Sec. 3.1) on tcgen05 tensor
 // cores (TMA-fed, accumulators in TMEM), the Gaussian modality score of eqs. (8)-(9) from the
 // same shared-memory X tiles, softmax, top-k, bin sums p_k = sum_{e in B_k} g_e, and the
-// per-(128-token tile, sample) partial sums of the joint table of eq. (12). The epilogue group
-// that completes the last partial of a sample reduces that sample's joint to P (eq. 13),
+// per-(128-token tile, sample) partial sums of the joint table of eq. (12). The reducer warp of the
+// CTA that completes the last partial of a sample reduces that sample's joint to P (eq. 13),
 // I (eq. 14) and the backward coefficient table; the one that completes the last sample writes
 // the loss of eq. (15). All reductions run in a fixed order: results are bitwise reproducible.
 //
@@ -145,8 +145,8 @@ __device__ __noinline__ float gauss_coef_pair(float2 mv, float2 mt, float2 vv, f
 // differences directly as well (see below). `red` is kMaxNV floats of shared scratch; the
 // sample's pieces [pb, pe) and token count n are passed in when already loaded (pb < 0: load).
 //
-// dry: the same instruction path with every global access and fence skipped. The first epilogue
-// warp runs it once while it waits for its first accumulator, so that this code, which a CTA
+// dry: the same instruction path with every global access and fence skipped. The reducer warp
+// runs it once while the first tile streams in, so that this code, which a CTA
 // otherwise runs once at the very end, is in the instruction cache when the last piece of a
 // sample arrives (a dry run must not touch memory: its loads would queue behind the X stream).
 __device__ __noinline__ void sample_reduce(const FwdParams& p, int s, float* red, int pb, int pe,
