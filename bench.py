@@ -141,8 +141,9 @@ def algorithmic(wl):
     return step_bytes, step_flops, fwd_bytes, bwd_bytes
 
 
-# Special-function unit: 16 exp2 results per SM and clock (4 per sub-partition), 152 SMs.
-SFU_PER_SM_CLK = 16
+# Special-function unit: 32 exp2 results per SM and clock (8 per sub-partition), from the attention
+# score's exponentials against the unit's utilisation counter.
+SFU_PER_SM_CLK = 32
 
 
 class ClockSampler:
@@ -741,7 +742,7 @@ def measure_next(bd, st, dev, flush, steps, hbm, tf_sus, sm_mhz, n_sms):
         pairs = float(aw.B) * aw.H * aw.S * (aw.S + 1) / 2.0
         flops = 4.0 * pairs * aw.hd                            # causal Q K^T and P V
         ach = flops / (ms * 1e-3) / 1e12
-        exp_peak = 16 * n_sms * sm_mhz * 1e-3                  # Gexp/s on the special-function unit
+        exp_peak = SFU_PER_SM_CLK * n_sms * sm_mhz * 1e-3                  # Gexp/s on the special-function unit
         out[f"attention_fwd_hkv{hkv}"] = {
             "us": 1e3 * ms, "bound": "tensor", "flops": flops, "achieved": ach, "peak": tf_sus,
             "unit": "TFLOP/s", "frac": ach / tf_sus, "exp_rate_frac": pairs / (ms * 1e-3) / 1e9 / exp_peak,
@@ -862,7 +863,7 @@ def main():
             ach = n_exp / (ms * 1e-3) / 1e9
             rooflines[name] = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Gexp/s",
                                "frac": ach / peak, "traffic": None, "kernel": "k_attn_mass",
-                               "peak_source": "derived: 16 exp2 per SM and clock x SMs x max SM clock"}
+                               "peak_source": "derived: 32 exp2 per SM and clock x SMs x max SM clock"}
         else:
             call = "fwd" if name.startswith("fwd") else "bwd"
             by = fwd_bytes if call == "fwd" else bwd_bytes
