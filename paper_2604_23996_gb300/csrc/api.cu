@@ -596,6 +596,7 @@ smoes_status smoes_attention_fwd(smoes_plan P, const smoes_attn_args* args, cons
   p.x_norm = a.x_norm;
   p.M = M;
   p.part = v.attn_part;
+  p.ticket = v.attn_ticket;
   p.status = v.status;
   p.n_qtiles = a.S / 128;
   p.n_items = a.B * a.H * p.n_qtiles;

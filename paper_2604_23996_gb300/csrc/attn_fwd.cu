@@ -356,6 +356,21 @@ __host__ __device__ inline AttnLayout attn_layout() {
   return L;
 }
 
+// M of a token from its heads' scores, in head order (eq. 3), optionally blended with the carried
+// score (eq. 4).
+__device__ __forceinline__ void average_heads(const AttnParams& p, int tok) {
+  float sum = 0.f;
+#pragma unroll 8
+  for (int hh = 0; hh < p.H; ++hh) sum += __ldcg(p.part + static_cast<size_t>(hh) * p.T + tok);
+  float mv = sum / static_cast<float>(p.H);
+  if (p.xattn_norm) {
+    const float an = __ldg(p.xattn_norm + tok), rn = __ldg(p.x_norm + tok);
+    const float mprev = p.m_prev ? __ldg(p.m_prev + tok) : static_cast<float>(__ldg(p.is_vision + tok) != 0);
+    mv = (an * mv + rn * mprev) / (an + rn);
+  }
+  reinterpret_cast<float2*>(p.M)[tok] = make_float2(mv, 1.f - mv);
+}
+
 template <bool kFloatM, int kTiles>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -386,6 +401,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   uint64_t* drain = bars + 30;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 31);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
+  int* last_head = abort_flag + 1;    // this CTA's head was its tile's last
   float* mxs = reinterpret_cast<float*>(base + L.mx);
   float* mrg = reinterpret_cast<float*>(base + L.mrg);
 
@@ -667,7 +683,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       if (!wait_bar(mrg_bar + t, nt & 1u, wc)) break;
       l = mb[row] + mb[2 * kAttnTile + row];               // in key order, the same in both halves
       const float il = 1.f / l;
-      if (hf == 0)                                         // head result (averaged by the next kernel)
+      if (hf == 0)                                         // head result
         p.part[static_cast<size_t>(w.h) * p.T + static_cast<size_t>(w.b) * p.S + q] = (a + mb[3 * kAttnTile + row]) * il;
       // O / l: half a row per thread
       if (!wait_bar(o_full + t, nt & 1u, wc)) break;
@@ -686,6 +702,26 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       tc_fence_before();
       mbar_arrive(o_empty + t);
     }
+    // One item per CTA: the tile's last head averages the heads here, in the warps that wrote this
+    // head's scores. Reached on every path out of the loop, so the barriers complete and the ticket
+    // is zero again for the next call also after a wait that ran out. A second launch made
+    // eager calls of 1 x 8 x 128, which the host bounds, slower than one kernel had been (13.3 ->
+    // 14.9 us; now 10.3-10.7 against 11.1). In a graph the ticket costs 0.4-0.8 us more than it.
+    if (kTiles == 1 && grp == 0) {
+      const AttnItem w = decode_item<kTiles>(p, dealt_item(0));
+      __syncwarp();
+      named_bar(1, 128);
+      if (row == 0) {
+        uint32_t* ticket = p.ticket + w.b * p.n_qtiles + w.qt0;
+        __threadfence();                       // the four warps' scores, ordered before it by the barrier
+        const bool last = atomicAdd(ticket, 1u) + 1u == static_cast<uint32_t>(p.H);
+        if (last) *ticket = 0u;
+        __threadfence();
+        *last_head = last ? 1 : 0;
+      }
+      named_bar(1, 128);
+      if (*last_head) average_heads(p, w.b * p.S + w.qt0 * kAttnTile + row);
+    }
   }
 
   // the role branches leave single lanes running on their own: the warp reconverges before
@@ -697,25 +733,14 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// M of a token from its heads' scores, in head order (eq. 3), optionally blended with the carried
-// score (eq. 4). A ticket per (sequence, query tile) taken at the end of every item instead, with
-// its fences, stopped the CTA for microseconds between items: 639 -> 607 us on 8 x 16 x 4096, 71 ->
-// 56 us on 16 x 32 x 256.
+// The heads' average of a call with more tiles than SMs: a ticket per (sequence, query tile) taken at
+// the end of every item instead, with its fences, stopped the CTA for microseconds between items:
+// 639 -> 607 us on 8 x 16 x 4096, 71 -> 56 us on 16 x 32 x 256.
 __global__ void __launch_bounds__(256) k_attn_average(const AttnParams p) {
   pdl_wait();                                  // the heads' scores of the kernel just before
   pdl_trigger();
   const int tok = blockIdx.x * 256 + threadIdx.x;
-  if (tok >= p.T) return;
-  float sum = 0.f;
-#pragma unroll 8
-  for (int hh = 0; hh < p.H; ++hh) sum += __ldcg(p.part + static_cast<size_t>(hh) * p.T + tok);
-  float mv = sum / static_cast<float>(p.H);
-  if (p.xattn_norm) {
-    const float an = __ldg(p.xattn_norm + tok), rn = __ldg(p.x_norm + tok);
-    const float mprev = p.m_prev ? __ldg(p.m_prev + tok) : static_cast<float>(__ldg(p.is_vision + tok) != 0);
-    mv = (an * mv + rn * mprev) / (an + rn);
-  }
-  reinterpret_cast<float2*>(p.M)[tok] = make_float2(mv, 1.f - mv);
+  if (tok < p.T) average_heads(p, tok);
 }
 
 }  // namespace
@@ -736,7 +761,7 @@ cudaError_t launch_attn_fwd(const AttnFwdParams& fp, const CUtensorMap& tmQ, con
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3(grid), dim3(kAttnThreads), smem, s, tmQ, tmK, tmV, fp);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || single) return e;   // (one item per CTA: averaged by its last head)
   return launch_pdl(k_attn_average, dim3((p.T + 255) / 256), dim3(256), 0, s, p);
 }
 

@@ -143,3 +143,29 @@ def test_forward_key_chunks_and_rescale(bd, B, H, Hkv, S, case):
                                                aw.key_bias.reshape(B, S))
     _check_O(Og, Oref, float(V.float().abs().max()), "O")
     assert_tensor_close(Mg[:, 0], mass.reshape(-1), "vision mass")
+
+
+@pytest.mark.parametrize("B,H,S", [(1, 8, 128), (3, 8, 384), (19, 8, 128), (10, 8, 256)])
+def test_forward_heads_averaged_on_repeated_calls(bd, B, H, S):
+    # up to 152 query tiles the tile's last head averages the heads (a ticket that every call leaves
+    # at zero, shared with the attention score's), with more a kernel of its own: one launch of each
+    # kind at the line (152 and 160 tiles), repeated on one workspace with the score in between
+    aw, K, V = _case(B, H, H, S, seed=40 + B, n_image=S // 4)
+    rng = np.random.default_rng(B)
+    m_prev = rng.random(B * S).astype(np.float32)
+    norms = [(0.5 + rng.random(B * S)).astype(np.float32) for _ in range(2)]
+    r, attn, _, M0 = _run(bd, aw, K, V, H, m_prev=m_prev, norms=norms)
+    _, mass = O.attention_forward_with_mass(aw.Q.double().numpy(), K.double().numpy(), V.double().numpy(),
+                                            m_prev.reshape(B, S).astype(np.float64), aw.sm_scale, True,
+                                            aw.key_bias.reshape(B, S))
+    an, xn = (n.astype(np.float64) for n in norms)
+    assert_tensor_close(M0[:, 0], (an * mass.reshape(-1) + xn * m_prev) / (an + xn), "blended score")
+    Vg, Ot = V.cuda(), torch.empty((B, H, S, 128), dtype=torch.bfloat16, device="cuda")
+    M, Ms = (torch.empty((B * S, 2), device="cuda") for _ in range(2))
+    for _ in range(3):
+        M.fill_(float("nan"))
+        assert bd.smoes_attention_fwd(r.plan, attn, Vg, H, Ot, M, r.ws) == 0
+        r.modality_score(bd.SMOES_SCORE_ATTN, Ms, attn=attn)
+        assert r.device_status()[0] == 0
+        np.testing.assert_array_equal(M.cpu().numpy(), M0)
+        assert_tensor_close(Ms.cpu().numpy(), M0, "score kernel")
