@@ -394,7 +394,8 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
   uint64_t* kt_empty = bars + 14;     // [kKtStages] count 16: a lane of every softmax warp
   uint64_t* s_full = bars + 16;       // [2] the tile's scores are in tensor memory
   uint64_t* mx_bar = bars + 18;       // [2] count 256: both halves' row maxima are written
-  uint64_t* p_full = bars + 20;       // [tile][half] count 128: 64 keys' weights are in tensor memory
+  uint64_t* p_full = bars + 20;       // [tile][half] count 128: 64 keys' weights are in tensor memory; half 0's
+                                      // also counts both halves' rescales of O (count 384)
   uint64_t* o_full = bars + 24;       // [2] the item's last P V has completed
   uint64_t* o_empty = bars + 26;      // [2] count 256: O has been read
   uint64_t* mrg_bar = bars + 28;      // [2] count 256: both halves' sums are written
@@ -418,7 +419,7 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
       mbar_init(v_full + t, 1);
       mbar_init(v_empty + t, 1);
       mbar_init(s_full + t, 1);
-      mbar_init(p_full + 2 * t, 128);
+      mbar_init(p_full + 2 * t, 384);
       mbar_init(p_full + 2 * t + 1, 128);
       mbar_init(o_full + t, 1);
       mbar_init(o_empty + t, 256);
@@ -649,6 +650,14 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
             }
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           }
+          // Each half rescales its own 64 columns of O, but the products of either half's weights add to
+          // all 128. Half 0's are issued first, on p_full[2 t], so both halves arrive there with their
+          // rescale done (or none needed): no product of block j reaches O before both rescales of
+          // block j. The arrival comes a weigh() ahead of half 0's own, so the MMA warp waits no longer
+          // for it. No thread can arrive for block j + 1 in the phase of block j: the scores of j + 1
+          // are issued after these products. (Block 0 has no rescale and is counted alike.)
+          tc_fence_before();
+          mbar_arrive(p_full + 2 * t);
           if (raise) m_used = m_new;
           // weights, in bf16 to the half's 32 columns of P; a row whose keys are all masked so far
           // has weights 0

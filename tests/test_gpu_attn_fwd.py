@@ -169,3 +169,32 @@ def test_forward_heads_averaged_on_repeated_calls(bd, B, H, S):
         assert r.device_status()[0] == 0
         np.testing.assert_array_equal(M.cpu().numpy(), M0)
         assert_tensor_close(Ms.cpu().numpy(), M0, "score kernel")
+
+
+@pytest.mark.parametrize("B,H,S", [(1, 2, 640), (4, 16, 640), (3, 28, 256)])
+@pytest.mark.parametrize("rows", ["all", "some", "even_tiles", "odd_tiles"])
+def test_forward_rescales_before_either_halfs_products(bd, B, H, S, rows):
+    # logits that grow by more than 2^8 with every key block, so that O is rescaled at every block: in
+    # every row, in every third row, or in one tile of each pair only. 10 query tiles take the kernel
+    # of one tile per item, 320 (with a pair of one) and 168 that of two. Each key half rescales its
+    # columns of O and both halves' products add to all of them: a product that came before the other
+    # half's rescale would differ from the oracle, or from call to call.
+    aw, K, V = _case(B, H, H, S, seed=500 + S + H, n_image=S // 4)
+    pos = np.arange(S)
+    on = {"all": pos >= 0, "some": pos % 3 == 1, "even_tiles": pos // 128 % 2 == 0, "odd_tiles": pos // 128 % 2 == 1}[rows]
+    aw.Q[..., 0] = torch.from_numpy(np.where(on, 16.0, 0.0)).to(torch.bfloat16)
+    K[..., 0] = torch.from_numpy(pos * (14.0 / 128) / (16.0 * aw.sm_scale)).to(torch.bfloat16)   # 14 nats a block
+    r, attn, Og, Mg = _run(bd, aw, K, V, H)
+    Oref, mass = O.attention_forward_with_mass(aw.Q.double().numpy(), K.double().numpy(), V.double().numpy(),
+                                               aw.is_vision.reshape(B, S).astype(np.float64), aw.sm_scale, True,
+                                               aw.key_bias.reshape(B, S))
+    _check_O(Og, Oref, float(V.float().abs().max()), "O")
+    assert_tensor_close(Mg[:, 0], mass.reshape(-1), "vision mass")
+    Vg = V.cuda()
+    first = torch.empty((B, H, S, 128), dtype=torch.bfloat16, device="cuda")
+    again, M1, M2 = torch.empty_like(first), torch.empty((B * S, 2), device="cuda"), torch.empty((B * S, 2), device="cuda")
+    assert bd.smoes_attention_fwd(r.plan, attn, Vg, H, first, M1, r.ws) == 0
+    for _ in range(50):
+        assert bd.smoes_attention_fwd(r.plan, attn, Vg, H, again, M2, r.ws) == 0
+        assert torch.equal(again.view(torch.int16), first.view(torch.int16)) and torch.equal(M1, M2)
+    assert r.device_status()[0] == 0
