@@ -57,19 +57,19 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, const W
   return mbar_try_wait(bar, parity) || wait_slow(bar, parity, w);
 }
 
-// Bounded wait of a role that runs ahead of the softmax warps: it sleeps between tries, which would
-// otherwise take issue slots from them (a third of all instructions).
+// Bounded wait of a whole warp that runs ahead of the softmax warps: it sleeps between tries, which
+// would otherwise take issue slots from them (a third of all instructions). Every lane returns the
+// same answer: full-warp shuffles and votes follow, and a lane that had left at the limit alone would
+// leave the others in them for good.
 __device__ __forceinline__ bool wait_idle(uint64_t* bar, uint32_t parity, const WaitCtx& w) {
-  if (mbar_try_wait(bar, parity)) return true;
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   const uint64_t t0 = global_ns();
   while (true) {
     __nanosleep(100);
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*w.abort_flag) return false;
-    if (global_ns() - t0 > w.limit_ns) {
-      raise_abort(w, 2u);
-      return false;
-    }
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const bool over = global_ns() - t0 > w.limit_ns;
+    if (over) raise_abort(w, 2u);
+    if (__any_sync(0xffffffffu, over || *w.abort_flag)) return false;
   }
 }
 
