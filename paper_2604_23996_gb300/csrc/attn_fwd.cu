@@ -105,6 +105,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
+// Largest bias (log2 units) that a chunk may add to its maximum's term instead of to every score. The
+// maximum is rounded at the bias's size, so the exponents f x + (g - max) can come out above 0 by half
+// an ulp of it: at most 64 below 2^31, far from overflow. A larger bias swallows the scores, as it does
+// in 64 bits from about 2^53: added to each, all of its keys weigh the same.
+constexpr float kMaxChunkBias = 2147483648.f;
+
 // What the keys of a 32-key chunk share. Labels and biases come in runs (an image, its text,
 // padding), so most chunks hold one value of each: then neither is read per key and thread (a
 // broadcast 16-byte load takes four cycles of the SM's shared-memory port; two per four keys
@@ -219,7 +225,8 @@ __device__ __forceinline__ void stage_key_terms(const AttnParams& p, int n_items
         c.bias = __shfl_sync(0xffffffffu, b[i], 0);
         c.m = __shfl_sync(0xffffffffu, m[i], 0);
         // (the maximum is then taken over the raw products: their factor has to be positive)
-        c.one_bias = __all_sync(0xffffffffu, __float_as_uint(b[i]) == __float_as_uint(c.bias)) && p.scale_log2 > 0.f;
+        const bool fits = fabsf(b[i]) < kMaxChunkBias || b[i] == -CUDART_INF_F;
+        c.one_bias = __all_sync(0xffffffffu, fits && __float_as_uint(b[i]) == __float_as_uint(c.bias)) && p.scale_log2 > 0.f;
         c.one_m = __all_sync(0xffffffffu, __float_as_uint(m[i]) == __float_as_uint(c.m));
         if (lane == 0) ch[i] = c;
       }

@@ -198,3 +198,27 @@ def test_forward_rescales_before_either_halfs_products(bd, B, H, S, rows):
         assert bd.smoes_attention_fwd(r.plan, attn, Vg, H, again, M2, r.ws) == 0
         assert torch.equal(again.view(torch.int16), first.view(torch.int16)) and torch.equal(M1, M2)
     assert r.device_status()[0] == 0
+
+
+@pytest.mark.parametrize("B,S,bias", [(1, 256, -1e30), (11, 256, -1e30), (1, 256, 1e30), (1, 256, 3e9), (11, 256, -1.4e9), (1, 256, -1e9)])
+@pytest.mark.parametrize("scale", [1.0, 30.0])
+def test_forward_one_bias_of_any_size_on_every_key(bd, B, S, bias, scale):
+    # left-padded prompts: every key that a padded query sees is masked by the same large finite bias.
+    # Past 2^53 the bias swallows the scores in 64 bits too and the row is a plain mean; a bias that the
+    # kernel keeps out of the scores (below 2^31 in log2 units) leaves the softmax of the scores. In
+    # between fp32 rounds the scores at the bias's size: the outputs then only have to be finite and
+    # within the values' range. Scores of up to 120 nats: none of it may overflow.
+    aw, K, V = _case(B, 8, 8, S, seed=77, n_image=S // 4)
+    aw.key_bias[:] = bias
+    aw.sm_scale *= scale
+    _, _, Og, Mg = _run(bd, aw, K, V, 8)
+    assert np.isfinite(Og).all() and np.isfinite(Mg).all()
+    Vmax = float(V.float().abs().max())
+    if 1.4e9 < abs(bias) < 1e16:
+        assert np.abs(Og).max() <= Vmax * (1 + 2.0 ** -7)
+        return
+    Oref, mass = O.attention_forward_with_mass(aw.Q.double().numpy(), K.double().numpy(), V.double().numpy(),
+                                               aw.is_vision.reshape(B, S).astype(np.float64), aw.sm_scale, True,
+                                               aw.key_bias.reshape(B, S))
+    _check_O(Og, Oref, Vmax, "O")
+    assert_tensor_close(Mg[:, 0], mass.reshape(-1), "vision mass")
