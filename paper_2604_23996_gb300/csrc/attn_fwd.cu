@@ -21,6 +21,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <atomic>
+
 #include "device_common.cuh"
 #include "ptx.cuh"
 #include "smoes_internal.cuh"
@@ -177,9 +179,12 @@ constexpr int kHalf = kAttnTile / 2;           // keys of a block per softmax gr
 // groups with a row's 128 keys per thread ran at 0.42 instructions per cycle.
 constexpr int kAttnThreads = 128 + 4 * 128;    // producer, MMA issuer, key terms, an idle warp, the groups
 // The launch's 640 x 96 registers dealt anew: 56 for the first four warps, 104 for the softmax warps
-// (128 x 56 + 512 x 104 = 60416 of 61440).
-__device__ __forceinline__ void attn_fewer_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 56;"); }
-__device__ __forceinline__ void attn_more_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 104;"); }
+// (128 x 56 + 512 x 104 = 60416 of 61440). setmaxnreg.inc waits without a limit for registers that the
+// launch does not hold, so the launch is refused if the kernel was compiled to fewer.
+constexpr int kFewerRegisters = 56, kMoreRegisters = 104;
+constexpr int kDealtRegisters = 128 * kFewerRegisters + (kAttnThreads - 128) * kMoreRegisters;
+__device__ __forceinline__ void attn_fewer_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFewerRegisters)); }
+__device__ __forceinline__ void attn_more_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kMoreRegisters)); }
 
 constexpr int kKtBlocks = 4;                   // key blocks per stage of key terms
 constexpr int kKtStages = 2;
@@ -772,11 +777,21 @@ cudaError_t launch_attn_fwd(const AttnFwdParams& fp, const CUtensorMap& tmQ, con
   const bool single = tiles <= n_sms;
   const int n_items = single ? tiles : ((p.n_qtiles + 1) / 2) * p.B * p.H;
   const int grid = n_items < n_sms ? n_items : n_sms;
-  auto k = p.m_prev ? (single ? k_attn_fwd<true, 1> : k_attn_fwd<true, 2>)
-                    : (single ? k_attn_fwd<false, 1> : k_attn_fwd<false, 2>);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  e = launch_pdl(k, dim3(grid), dim3(kAttnThreads), smem, s, tmQ, tmK, tmV, fp);
+  auto launch = [&](auto k, std::atomic<int>& regs) -> cudaError_t {
+    int held = regs.load(std::memory_order_relaxed);    // a constant of the build, asked for once
+    if (held == 0) {
+      cudaFuncAttributes fa;
+      const cudaError_t e = cudaFuncGetAttributes(&fa, k);
+      if (e != cudaSuccess) return e;
+      regs.store(held = fa.numRegs, std::memory_order_relaxed);
+    }
+    if (held * kAttnThreads < kDealtRegisters) return cudaErrorInvalidConfiguration;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return e != cudaSuccess ? e : launch_pdl(k, dim3(grid), dim3(kAttnThreads), smem, s, tmQ, tmK, tmV, fp);
+  };
+  static std::atomic<int> regs[4];
+  const cudaError_t e = p.m_prev ? (single ? launch(k_attn_fwd<true, 1>, regs[0]) : launch(k_attn_fwd<true, 2>, regs[1]))
+                                 : (single ? launch(k_attn_fwd<false, 1>, regs[2]) : launch(k_attn_fwd<false, 2>, regs[3]));
   if (e != cudaSuccess || single) return e;   // (one item per CTA: averaged by its last head)
   return launch_pdl(k_attn_average, dim3((p.T + 255) / 256), dim3(256), 0, s, p);
 }
