@@ -341,9 +341,11 @@ smoes_status smoes_plan_create(const smoes_router_desc* desc, smoes_plan* out) {
   P->bwd_tiles = (T + kBwdBT - 1) / kBwdBT;
   if (d.dtype == SMOES_BF16) {
     const int E_pad = round_up(E, 64);
-    // 256 columns per slice: with 512 (which fits at E <= 64) twice the token groups write partial
-    // dW, and d = 1280 leaves a half-empty slice (small_hidden step 101.0 -> 98.1 us, dsmoe_vlm backward
-    // 37.9 -> 37.7); with 128 at E = 128 every dz image is read twice as often (316 -> 367 us)
+    // 256 columns per slice. With 512, which fit at E <= 64, twice the token groups write partial dW, and
+    // d = 1280 leaves a half-empty slice (us, 512 -> 256 columns, E = 64): 2048 x 2048 17.9 -> 15.4, 16384 x
+    // 1024 28.3 -> 24.9, 16384 x 2048 38.0 -> 36.9, small_hidden's step 100.0 -> 97.5. The other way
+    // where 256 leaves more CTAs idle: 16384 x 4096 60.6 -> 61.2 (144 CTAs), 5120 71.7 -> 73.9 (140), 8192
+    // 108.4 -> 112.6 (128). With 128 at E = 128 every dz image is read twice as often (316 -> 367).
     const int dround = round_up(d.d, kBwdBD);
     P->bwd_slice_width = std::min(256, dround);
     P->bwd_slices = (dround + P->bwd_slice_width - 1) / P->bwd_slice_width;

@@ -365,11 +365,17 @@ struct BwdLayout {
   uint32_t wsl, dz, xst, stg, bars, total;
 };
 
-// dX^T accumulators in TMEM: kDxBufs buffers of 64 columns after the dW^T blocks (which take at
-// most 256 columns: two 128-column d-blocks of at most 128 experts), drained by two warp groups in turn.
+// dX^T accumulators in TMEM: kDxBufs buffers of 64 columns after the dW^T blocks (which take 256
+// columns: two 128-column d-blocks of 128 experts, or of 64 experts twice), drained by two warp groups
+// in turn.
 constexpr int kDxBufs = 4;
 constexpr int kDrainGroups = 2;
 constexpr int kBwdThreads = 64 + kDrainGroups * 128;
+// dW^T accumulators per d-block, taken by a CTA's tiles in turn and added at the end: the tensor cores
+// truncate an fp32 accumulator at every instruction, so its error grows with the tokens that it sums.
+// At E_pad = 64 a second one fits. Error of dW against the 64-bit product of the same dz, E = 64:
+// 131072 x 2048 1.61e-5 with one, 8.1e-6 with two; 65536 x 1280 5.2e-6, 2.6e-6. Time unchanged.
+__host__ __device__ constexpr int bwd_accs(int E_pad) { return E_pad <= 64 ? 2 : 1; }
 
 __host__ __device__ inline BwdLayout bwd_layout(int E_pad, int slice_width, int n_xst) {
   BwdLayout L;
@@ -424,6 +430,7 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const bool want_dx = p.dX != nullptr;
   constexpr uint32_t dz_half = static_cast<uint32_t>(E_pad) * 128u;         // one of hi / lo
   constexpr uint32_t dz_buf_bytes = 2u * dz_half;                           // hi + lo
+  constexpr int kAccs = bwd_accs(E_pad);
   WaitCtx wc{abort_flag, p.ws.status, p.limit_ns};
 
   if (threadIdx.x == 0) {
@@ -530,14 +537,14 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (!warp_wait(xfull + st, ph, wc)) { ok = false; break; }
         tc_fence_after();
         const uint32_t xs = xst0 + static_cast<uint32_t>(st) * 16384u;
-        const uint32_t dwc = tmem + static_cast<uint32_t>(b * E_pad);
+        const uint32_t dwc = tmem + static_cast<uint32_t>((2 * (lt % kAccs) + b) * E_pad);
         if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < kBwdBT / 16; ++ks) {     // K = 16 tokens per instruction
             const uint64_t da = sdesc_sw128(xs + ks * 2048, 8192, 1024);
             const uint64_t dh = sdesc_sw128(hi + ks * 2048, 8192, 1024);
             const uint64_t dl = sdesc_sw128(lo + ks * 2048, 8192, 1024);
-            umma_bf16(dwc, da, dh, id_dw, (lt > 0 || ks > 0) ? 1u : 0u);
+            umma_bf16(dwc, da, dh, id_dw, (lt >= kAccs || ks > 0) ? 1u : 0u);
             umma_bf16(dwc, da, dl, id_dw, 1u);
           }
           umma_commit(xempty + st);             // the X stage is free once these MMAs complete
@@ -648,6 +655,12 @@ k_router_bwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         for (int c = 0; c < E_pad / 32; ++c) {
           float v[32];
           tmem_ld32(ta + 32u * c, v);
+          if (kAccs == 2 && grp + G < p.n_tiles) {         // (a CTA of one tile has not used the second)
+            float w[32];
+            tmem_ld32(ta + 2u * E_pad + 32u * c, w);
+#pragma unroll
+            for (int q = 0; q < 32; ++q) v[q] += w[q];
+          }
 #pragma unroll
           for (int q = 0; q < 32; ++q) {
             const int e = c * 32 + q;

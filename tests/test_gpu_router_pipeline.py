@@ -2,6 +2,7 @@
 every length of the top-k networks, one tile per CTA at the widest gate, CTAs that hand many
 samples to their reducer warp, two tiles per CTA with the permutation in the same launch, and
 backward slices whose last 64-column box starts past the hidden size."""
+import numpy as np
 import pytest
 import torch
 
@@ -39,3 +40,31 @@ def test_router_pipeline(bd, T, d, E, k, K, samples):
     wl = random_router_case(T + k, T, d, E, k, K, _lengths(T, samples), aligned=True)
     g = run_gpu(wl, bd, fused=True)
     compare(wl, g, run_oracle(wl))
+
+
+@pytest.mark.parametrize("T,d,E,k,K", [(65536, 2048, 64, 6, 8), (65536, 1280, 48, 4, 6), (131072, 512, 32, 4, 8)])
+def test_dw_error_of_the_accumulators(bd, T, d, E, k, K):
+    # dW against the 64-bit product of the operands that the tensor cores get: dz as bf16 hi + lo and X.
+    # What is left is the truncation of the fp32 accumulators, half an ulp (2^-25 .. 2^-24 of the
+    # accumulator) per instruction on average. A sum over random tokens grows like the square root, 2/3
+    # of its final size on average, so n instructions leave at most n 2^-25. A CTA's tiles (64 tokens,
+    # four K steps, hi and lo) go to two accumulators in turn; with one the error is twice as large.
+    g = torch.Generator(device="cuda").manual_seed(T + d)
+    X = torch.randn((T, d), generator=g, device="cuda").to(torch.bfloat16)
+    W = (0.02 * torch.randn((E, d), generator=g, device="cuda")).to(torch.bfloat16)
+    r = bd.Router(T, d, E, k, K, [0, T], np.arange(E) // (E // K))
+    r.forward(X, W, mu=0.05 * torch.randn((2, d), generator=g, device="cuda"), var=torch.ones((2, d), device="cuda"))
+    dW, dz = torch.empty((E, d), device="cuda"), torch.empty((T, E), device="cuda")
+    r.backward(X, W, r.M, dW, dlogits=dz, d_topk_w=1e-3 * torch.randn((T, k), generator=g, device="cuda"))
+    assert r.device_status()[0] == 0
+    hi = dz.to(torch.bfloat16)
+    lo = (dz - hi.float()).to(torch.bfloat16)
+    ref = torch.zeros((E, d), dtype=torch.float64, device="cuda")
+    for s in range(0, T, 8192):
+        ref += (hi[s:s + 8192].double() + lo[s:s + 8192].double()).T @ X[s:s + 8192].double()
+    groups = torch.cuda.get_device_properties(0).multi_processor_count // -(-d // 256)
+    tiles = -(-(T // 64) // groups)
+    n = -(-tiles // 2) * 4 * 2
+    err = float((dW.double() - ref).norm() / ref.norm())
+    assert err <= n * 2.0 ** -25, f"{err:.3g} > {n * 2.0 ** -25:.3g}"
+    print(f"{T} x {d}, E = {E}: {err:.2e}, {n} instructions per accumulator: at most {n * 2.0 ** -25:.2e}")
