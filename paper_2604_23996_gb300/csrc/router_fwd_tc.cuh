@@ -98,12 +98,6 @@ __device__ __forceinline__ void topk_merge(float (&tk)[L], const float (&v)[L]) 
       if ((i & j) == 0) cmp_desc(tk[i], tk[i + j]);
   }
 }
-// 2^x on the special-function unit: exp2f's value, without its scaling of results below 2^-126.
-__device__ __forceinline__ float ex2_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // The keys of 16 logits (experts 16 c + t) into the running list.
 template <int L>
@@ -533,7 +527,7 @@ __device__ void epilogue_tile(const FwdParams& p, const Src& src, const Release&
       float v[16];
       src.load16(c, v);
 #pragma unroll
-      for (int t = 0; t < 16; ++t) v[t] = ex2_ftz(fmaf(v[t], kLog2e, -mxl));   // saved e = exp(z - max)
+      for (int t = 0; t < 16; ++t) v[t] = exp2f(fmaf(v[t], kLog2e, -mxl));   // saved e = exp(z - max)
       emit(c, v);
     }
   }

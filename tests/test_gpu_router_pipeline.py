@@ -68,3 +68,26 @@ def test_dw_error_of_the_accumulators(bd, T, d, E, k, K):
     err = float((dW.double() - ref).norm() / ref.norm())
     assert err <= n * 2.0 ** -25, f"{err:.3g} > {n * 2.0 ** -25:.3g}"
     print(f"{T} x {d}, E = {E}: {err:.2e}, {n} instructions per accumulator: at most {n * 2.0 ** -25:.2e}")
+
+
+@pytest.mark.parametrize("E,K,dtype", [(64, 8, torch.bfloat16), (128, 16, torch.bfloat16), (72, 8, torch.bfloat16), (32, 4, torch.float32)])
+def test_scores_far_below_the_row_maximum_are_kept(bd, E, K, dtype):
+    # logits of 0, -60, -88 and -98 by bin: the last two bins' scores lie at 2^-127 and 2^-141, below
+    # the normal range, where fp32 still has steps of 2^-149. Scores, sums and products are each off by
+    # at most a step: bin sums of N_B scores by N_B / 2 steps and the rounding of the product.
+    T, d, k = 160, 64, 2
+    X = torch.zeros((T, d), dtype=dtype, device="cuda")
+    X[:, 0] = 1.0
+    eb = np.arange(E) // (E // K)
+    depth = torch.tensor([0.0, -60.0, -88.0, -98.0])[torch.from_numpy(eb % 4)]
+    W = torch.zeros((E, d), dtype=dtype, device="cuda")
+    W[:, 0] = depth.to(dtype).cuda()
+    r = bd.Router(T, d, E, k, K, [0, T], eb, bd.SMOES_F32 if dtype == torch.float32 else bd.SMOES_BF16)
+    M = torch.full((T, 2), 0.5, device="cuda")
+    r.forward(X, W, M_in=M)
+    g = torch.softmax(depth.double(), dim=0).numpy()
+    ref = np.array([g[eb == b].sum() for b in range(K)])
+    got = r.bin_prob.cpu().numpy()
+    step = 2.0 ** -149
+    np.testing.assert_allclose(got, np.tile(ref, (T, 1)), rtol=2e-5, atol=(E // K / 2 + 1) * step)
+    assert (got[:, eb[::E // K] % 4 == 3] > 0).all()
