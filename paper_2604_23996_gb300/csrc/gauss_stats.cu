@@ -35,15 +35,26 @@ constexpr uint32_t kStatStageBytes = 32768;      // rows of one stage: as many a
 constexpr uint32_t kStatMergeBytes = kStatConsumers * 8u * 4u * 4u;   // (s1, s2) x (v, t) per thread
 constexpr int kStatMaxRows = 16384;              // rows per block (their labels stay in shared memory)
 
-// x / n with the reciprocal formed once: GB300 has two fp64 FMAs per SM and clock, and one fp64
-// division per feature and thread cost 20 us of the pass over d = 2048. Where the reciprocal
-// overflows (n = 0 or subnormal) the division itself is taken.
-__device__ __forceinline__ double div_by(double x, double n, double inv) {
-  return isfinite(inv) ? x * inv : x / n;
+// x / n with the reciprocal formed once: GB300 has two fp64 FMAs per SM and clock, and an fp64 division
+// takes many. The product is off by up to two ulp: enough for what is rounded to fp32 (one division per
+// feature and thread for the shift cost 20 us of the pass over d = 2048). For what enters the fp64
+// state its remainder, exact as an FMA, corrects it to the division's own rounding (Markstein's theorem
+// on the correctly rounded reciprocal). Where the reciprocal leaves the normal range (n = 0 or
+// subnormal) the division itself is taken; an infinite quotient has no remainder.
+__device__ __forceinline__ bool has_inverse(double inv) {   // a normal number (its exponent bits: fp64 compares are slow too)
+  return ((static_cast<uint32_t>(__double2hiint(inv)) >> 20 & 0x7ffu) - 1u) < 2046u;
 }
-// Shift of a feature, the same in both kernels: the previous mean in fp32, 0 for an empty state.
+__device__ __forceinline__ float div_f32(double x, double n, double inv) {
+  return static_cast<float>(has_inverse(inv) ? x * inv : x / n);
+}
+__device__ __forceinline__ double div_f64(double x, double n, double inv) {
+  if (!has_inverse(inv)) return x / n;
+  const double q = x * inv, r = fma(-q, n, x);
+  return isfinite(r) ? fma(r, inv, q) : q;
+}
+// Shift of a feature, the same in both kernels: the previous mean to fp32 precision, 0 for an empty state.
 __device__ __forceinline__ float stat_shift(double n, double inv, double s_mu) {
-  return n > 0.0 ? static_cast<float>(div_by(s_mu, n, inv)) : 0.f;
+  return n > 0.0 ? div_f32(s_mu, n, inv) : 0.f;
 }
 
 // Eight consecutive features of a staged row as four packed pairs.
@@ -301,7 +312,7 @@ __global__ void __launch_bounds__(kFinSlices * kFinCols) k_stats_finalize(const 
   }
   if (sl == 0) {                                  // (one warp of the block: fp64 is scarce)
     inv_N0 = 1.0 / N0;
-    mean0 = div_by(Smu0, N0, inv_N0);             // S_mu,t-1 / N_t-1 (used when N0 > 0)
+    mean0 = div_f64(Smu0, N0, inv_N0);             // S_mu,t-1 / N_t-1 (used when N0 > 0)
   }
   red[0][sl][col] = a1;
   red[1][sl][col] = a2;
@@ -321,20 +332,20 @@ __global__ void __launch_bounds__(kFinSlices * kFinCols) k_stats_finalize(const 
   const double inv_N1 = 1.0 / N1;
   if (n > 0.0) {
     const double c = static_cast<double>(stat_shift(N0, inv_N0, Smu0));
-    const double db = s1 * inv_n;                                     // batch mean - c
+    const double db = div_f64(s1, n, inv_n);                          // batch mean - c
     const double m2 = fmax(s2 - s1 * db, 0.0);                        // sum (x - mu_b)^2
     Smu1 += n * (c + db);                                             // eq. (6)
     Svar1 += m2;                                                      // eq. (7)
     if (N0 > 0.0) {
       const double dm = (c - mean0) + db;                             // mu_b - S_mu,t-1 / N_t-1
-      Svar1 += dm * dm * (beta * N0 * n * inv_N1);
+      Svar1 += dm * dm * div_f64(beta * N0 * n, N1, inv_N1);
     }
   }
   p.S_mu[at] = Smu1;
   p.S_var[at] = Svar1;
   if (i == 0) p.N[m] = N1;
-  if (p.mu_out) p.mu_out[at] = static_cast<float>(div_by(Smu1, N1, inv_N1));
-  if (p.var_out) p.var_out[at] = static_cast<float>(div_by(Svar1, N1, inv_N1));
+  if (p.mu_out) p.mu_out[at] = div_f32(Smu1, N1, inv_N1);
+  if (p.var_out) p.var_out[at] = div_f32(Svar1, N1, inv_N1);
 }
 
 // Eqs. (10)-(11) and the stable ascending rank of f_spec; one thread per expert.

@@ -120,6 +120,34 @@ def test_first_update_gives_the_batch_moments(bd):
     assert N.cpu().numpy().tolist() == [float((wl.is_vision == 1).sum()), float((wl.is_vision == 0).sum())]
 
 
+@pytest.mark.parametrize("T,d", [(3001, 256), (777, 2056)])
+def test_stats_means_are_rounded_as_divisions(bd, T, d):
+    # features on a grid whose fp32 sums are exact, from the empty state: S_mu is then n (s / n) with two
+    # fp64 roundings, and the mean that leaves is S_mu / n rounded to fp32
+    g = torch.Generator(device="cuda").manual_seed(T)
+    X = (torch.randint(-64, 64, (T, d), generator=g, device="cuda") / 8.0).to(torch.bfloat16)
+    v = (torch.arange(T, device="cuda") % 3 == 0).to(torch.uint8)
+    r = _plan(bd, T, d, torch.bfloat16)
+    N = torch.zeros(2, dtype=torch.float64, device="cuda")
+    S_mu, S_var = (torch.zeros((2, d), dtype=torch.float64, device="cuda") for _ in range(2))
+    mu, var = (torch.empty((2, d), device="cuda") for _ in range(2))
+    assert bd.smoes_gaussian_stats_update(r.plan, X, v, 0.99, N, S_mu, S_var, mu, var, r.ws) == 0
+    for m in range(2):
+        rows = X[v == 1 - m].double().cpu().numpy()
+        n = float(len(rows))
+        assert N[m].item() == n
+        np.testing.assert_array_equal(S_mu[m].cpu().numpy(), n * (rows.sum(axis=0) / n))
+        np.testing.assert_array_equal(mu[m].cpu().numpy(), (S_mu[m].cpu().numpy() / n).astype(np.float32))
+    # infinite and NaN features stay in their column and leave the others alone
+    keep = S_mu.clone()
+    X[5, 8], X[7, 16] = float("inf"), float("nan")
+    N.zero_(), S_mu.zero_(), S_var.zero_()
+    assert bd.smoes_gaussian_stats_update(r.plan, X, v, 0.99, N, S_mu, S_var, mu, var, r.ws) == 0
+    bad = torch.zeros((2, d), dtype=torch.bool, device="cuda")
+    bad[1, 8] = bad[1, 16] = True
+    assert torch.equal(S_mu[~bad], keep[~bad]) and S_mu[1, 8].item() == float("inf") and torch.isnan(S_mu[1, 16])
+
+
 def _bins_steps(bd, E, n_bins, counts_seq, beta):
     dev = "cuda"
     r = bd.Router(128, 64, E, 2, n_bins, [0, 128], np.arange(E) // (E // n_bins))
