@@ -872,7 +872,10 @@ __global__ void __launch_bounds__(kDwSlices * kDwCols) k_dw_reduce(const BwdPara
 
 cudaError_t launch_dz_prep(const BwdParams& p, cudaStream_t s) {
   const int E_pad = round_up(p.dm.E, 64);
-  const int blocks = p.n_tiles < 4 * p.n_sms ? p.n_tiles : 4 * p.n_sms;   // (64 registers: four per SM)
+  // Four blocks per SM: what the plain variants' 64 registers allow. The others take 80 to 128, so an SM
+  // holds two or three of them and starts the rest as those end; a grid of just what it holds was no
+  // better (131072 x 1024, E = 64, upstream gradient 127.3 -> 125.4 us; 65536 x 1024, E = 128 94.5 -> 96.0).
+  const int blocks = p.n_tiles < 4 * p.n_sms ? p.n_tiles : 4 * p.n_sms;
   // the upstream-gradient and balance variants keep their tables out of the common kernel's
   // registers; the balance variant still checks the arming flag on the device
   const bool up = p.d_topk_w != nullptr, bal = p.balance_armed != 0;

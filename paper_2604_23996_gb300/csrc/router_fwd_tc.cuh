@@ -1290,7 +1290,8 @@ k_router_fwd_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
 }
 
-// Top-k insertion width: k rounded up to 2, 4, 6, 8 or 16.
+// Length of the top-k arrays: k rounded up to 2, 4, 6, 8 or 16 (the sorting networks run on 2, 4, 8 or 16
+// keys, so 6 shares those of 8 and saves two outputs).
 template <class F>
 cudaError_t dispatch_km(int k, F&& f) {
   if (k <= 2) return f(std::integral_constant<int, 2>());
