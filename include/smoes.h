@@ -305,7 +305,8 @@ smoes_status smoes_bin_permute(smoes_plan plan, const int32_t* topk_idx, const i
  *   statistics the next score uses; NaN for a modality never seen).
  *   The batch sums are shifted by the previous mean (exact algebra, no cancellation); partial
  *   sums are fp32 per block of rows and fp64 across blocks, in a fixed order (reproducible).
- *   ws: the plan's workspace (per-block partial sums). */
+ *   ws: the plan's workspace (per-block partial sums). After a bounded wait that ran out
+ *   (SMOES_ERR_DEVICE_TIMEOUT) the state, mu and var are left as they were. */
 smoes_status smoes_gaussian_stats_update(smoes_plan plan, const void* X, const uint8_t* is_vision,
                                          double beta, double* N, double* S_mu, double* S_var,
                                          float* mu, float* var, void* ws, size_t ws_bytes,

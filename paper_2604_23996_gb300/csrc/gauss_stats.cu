@@ -74,8 +74,8 @@ __device__ __forceinline__ void staged8(const uint8_t* row, int f, uint64_t (&x)
 }
 
 // Block b sums rows [b T / G, (b+1) T / G). part: [G][4][d] = (s1_v, s2_v, s1_t, s2_t);
-// nvis: [G] vision rows of the block; block 0 also keeps a copy of N_{t-1} for the finalize
-// kernel (which overwrites N).
+// nvis: [G] vision rows of the block, -1 after a wait that ran out; block 0 also keeps a copy of N_{t-1}
+// for the finalize kernel (which overwrites N).
 //
 // Bound by HBM. Rows are contiguous, so one thread streams them into a ring of four 32 KB stages
 // with bulk copies (up to 128 KB in flight per SM, against the 64 KB of register loads of two
@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kStatThreads, 1) k_stats_partial(const StatsPa
       WaitCtx wd = wc;                             // every issued copy lands before the block exits
       int dummy = 0;
       wd.abort_flag = &dummy;
+      if (wd.limit_ns < kWaitLimitNs) wd.limit_ns = kWaitLimitNs;   // (whatever the plan's own limit)
       for (long q = (issued > kStatStages ? issued - kStatStages : 0); q < issued; ++q)
         mbar_wait(full + (q % kStatStages), static_cast<uint32_t>((q / kStatStages) & 1), wd);
     }
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(kStatThreads, 1) k_stats_partial(const StatsPa
       const uint32_t row_bytes = static_cast<uint32_t>(w * es);
       for (int j0 = r0; j0 < r1; j0 += R) {
         const int nr = min(R, r1 - j0);
-        if (!ok || !mbar_wait(full + st, ph, wc)) { ok = false; break; }
+        if (!ok || !warp_wait(full + st, ph, wc)) { ok = false; break; }
         if (act) {
           const uint8_t* rows = ring + st * kStatStageBytes;
           const uint8_t* lb = lab + (j0 - r0);
@@ -249,6 +250,10 @@ __global__ void __launch_bounds__(kStatThreads, 1) k_stats_partial(const StatsPa
       named_bar(1, kStatConsumers);                // merge is rewritten by the next pass
     }
   }
+  // a block whose wait ran out has no sums: its count says so, and the state stays as it was
+  __syncwarp();
+  __syncthreads();
+  if (threadIdx.x == 0 && *wc.abort_flag) p.nvis[b] = -1;
 }
 
 // One (modality, feature) column per (block column, 16 slices): slice t sums the partials of
@@ -304,11 +309,16 @@ __global__ void __launch_bounds__(kFinSlices * kFinCols) k_stats_finalize(const 
   }
   if (sl == kFinSlices - 1) {                     // |T_v|: integer counts, lanes stride the blocks
     int nvis = 0;
-    for (int g = col; g < G; g += 32) nvis += p.nvis[g];
+    bool out = false;                             // a block has no sums
+    for (int g = col; g < G; g += 32) {
+      nvis += p.nvis[g];
+      out = out || p.nvis[g] < 0;
+    }
     nvis = __reduce_add_sync(0xffffffffu, nvis);
+    out = __any_sync(0xffffffffu, out);
     const int cnt = col == 0 ? nvis : p.T - nvis;
     if (col < 2) inv_n_s[col] = cnt > 0 ? 1.0 / cnt : 0.0;
-    if (col == 0) cnt_s = nvis;
+    if (col == 0) cnt_s = out ? -1 : nvis;
   }
   if (sl == 0) {                                  // (one warp of the block: fp64 is scarce)
     inv_N0 = 1.0 / N0;
@@ -317,7 +327,7 @@ __global__ void __launch_bounds__(kFinSlices * kFinCols) k_stats_finalize(const 
   red[0][sl][col] = a1;
   red[1][sl][col] = a2;
   __syncthreads();
-  if (sl != 0 || i2 >= 2 * p.d) return;
+  if (sl != 0 || i2 >= 2 * p.d || cnt_s < 0) return;
   double s1 = 0.0, s2 = 0.0;
 #pragma unroll
   for (int t = 0; t < kFinSlices; ++t) {
