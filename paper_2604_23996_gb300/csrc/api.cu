@@ -546,7 +546,6 @@ smoes_status smoes_modality_score(smoes_plan P, smoes_score_mode mode, const smo
     p.ticket = v.attn_ticket;
     p.status = v.status;
     p.n_qtiles = (a.S + 127) / 128;
-    p.n_items = a.B * p.n_qtiles * a.H;
     p.limit_ns = P->limit_ns;
     CUtensorMap tq, tk;
     const uint64_t rows = static_cast<uint64_t>(a.B) * a.H * a.S;
@@ -601,7 +600,6 @@ smoes_status smoes_attention_fwd(smoes_plan P, const smoes_attn_args* args, cons
   p.ticket = v.attn_ticket;
   p.status = v.status;
   p.n_qtiles = a.S / 128;
-  p.n_items = a.B * a.H * p.n_qtiles;
   p.limit_ns = P->limit_ns;
   fp.Hkv = n_kv_heads;
   fp.O = O;

@@ -4,20 +4,20 @@
 // query head h reads key/value head h / (H / H_kv).
 //
 // A work item is (sequence, head, pair of adjacent 128-query tiles); the tiles share one stream of
-// 128-key blocks. Roles: a TMA producer, an MMA issuer, a warp that stages the keys' bias and
-// carried score, and four softmax groups of four warps, one per tile
-// and half of a block's keys, a query row per thread. For each block S = Q K^T goes to tensor
-// memory; the row's two threads exchange their maxima, form the weights and keep the normaliser
-// l = sum 2^(x - max) and the vision mass a = sum 2^(x - max) m (fp32, packed pairs). The weights return to tensor memory as bf16 over the scores they came from and are
-// the A operand of O += P V. The maximum in use is raised only when a block's maximum exceeds it by
-// more than 2^8 (then l, a and O are rescaled), so rescales are rare.
+// 128-key blocks. Roles: a TMA producer, an MMA issuer, a warp that stages the keys' bias and carried
+// score, and four softmax groups of four warps, one per tile and half of a block's keys, a query row
+// per thread. For each block S = Q K^T goes to tensor memory; the row's two threads exchange their
+// maxima, form the weights and keep the normaliser l = sum 2^(x - max) and the vision mass
+// a = sum 2^(x - max) m (fp32, packed pairs). The weights return to tensor memory as bf16 over the
+// scores they came from and are the A operand of O += P V. The maximum in use is raised only when a
+// block's maximum exceeds it by more than 8 (a factor of 2^8; then l, a and O are rescaled).
 //
-// Bound by the tensor pipe (two 128 x 128 x 128 products per tile and block) once the two tiles
-// hide each other's softmax: with the weights in tensor memory nothing but Q, K and V needs
-// shared memory, and S, P and O of two tiles fill the 512 columns. One tile per CTA, its weights
-// in shared memory, had every step of a block wait for the one before: 8 x 16 x 4096 causal with
-// H_kv = 4 took 1270 us, now 556 us (607 us before the converged issue). Groups of a whole row (128 keys per thread, half the warps)
-// took 735 us with the scores in registers and 643 us reading them twice.
+// Bound by a tile's chain S -> softmax -> P V, which the other tile's hides in part. With the weights
+// in tensor memory no P tile takes shared memory, and S, P and O of two tiles fill the 512 columns. One
+// tile per CTA, its weights in shared memory, had every step of a block wait for the one before: 8 x 16 x
+// 4096 causal with H_kv = 4 took 1270 us, now 560 (607 before the converged issue). Groups of a whole
+// row (128 keys per thread, half the warps) took 735 us with the scores in registers and 643 us reading
+// them twice. A vote in the softmax warps' waits, as the other roles have: 566 us, 1 x 16 x 512 16.1 -> 17.3.
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -725,9 +725,10 @@ k_attn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUte
     }
     // One item per CTA: the tile's last head averages the heads here, in the warps that wrote this
     // head's scores. Reached on every path out of the loop, so the barriers complete and the ticket
-    // is zero again for the next call also after a wait that ran out. A second launch made
-    // eager calls of 1 x 8 x 128, which the host bounds, slower than one kernel had been (13.3 ->
-    // 14.9 us; now 10.3-10.7 against 11.1). In a graph the ticket costs 0.4-0.8 us more than it.
+    // is zero again for the next call also after a wait that ran out. With a second launch instead,
+    // eager calls of 1 x 8 x 128 (3000 in a row), which the host bounds, take 12.0-13.8 us against
+    // 9.9-11.1 (10.1-11.7 before this kernel had two tiles per item); in a graph the ticket costs 0.3 us
+    // of 8.1 there and 0.1 of 15.6 at 1 x 16 x 512 (9.3 and 17.1 before).
     if (kTiles == 1 && grp == 0) {
       const AttnItem w = decode_item<kTiles>(p, dealt_item(0));
       __syncwarp();

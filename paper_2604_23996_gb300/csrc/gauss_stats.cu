@@ -82,7 +82,7 @@ __device__ __forceinline__ void staged8(const uint8_t* row, int f, uint64_t (&x)
 // 256-thread blocks that stopped while they summed), and 512 threads sum: w / 8 threads per row
 // (rounded to warps), the rows of a stage dealt to 512 / that groups, whose sums are added in group
 // order at the end. Packed fp32 pairs: three instructions per two features.
-// 131072 x 2048 bf16, both kernels: 150.7 -> 93.2 us (5.8 TB/s of X).
+// 131072 x 2048 bf16, both kernels: 150.6 -> 92.6 us (5.8 TB/s of X).
 template <bool kBf16>
 __global__ void __launch_bounds__(kStatThreads, 1) k_stats_partial(const StatsParams p) {
   extern __shared__ __align__(128) uint8_t st_smem[];

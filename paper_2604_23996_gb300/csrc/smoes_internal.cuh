@@ -193,7 +193,6 @@ struct AttnParams {
   uint32_t* ticket;          // [B * n_qtiles]
   uint32_t* status;
   int n_qtiles;
-  int n_items;
   uint64_t limit_ns;
 };
 

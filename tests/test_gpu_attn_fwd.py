@@ -121,9 +121,12 @@ def test_attention_forward_limits(bd):
 
 
 @pytest.mark.parametrize("B,H,Hkv,S,case", [(1, 2, 1, 640, "rising"), (3, 8, 8, 128, "padded"), (20, 16, 16, 256, "runs"),
-                                            (1, 4, 4, 384, "scattered"), (1, 2, 2, 256, "negative")])
+                                            (1, 4, 4, 384, "scattered"), (1, 2, 2, 256, "negative"),
+                                            (4, 16, 4, 384, "rising"), (10, 16, 16, 128, "padded"), (5, 16, 8, 384, "scattered"),
+                                            (6, 16, 16, 256, "negative")])
 def test_forward_key_chunks_and_rescale(bd, B, H, Hkv, S, case):
-    # an odd number of query tiles (a pair of one), many short items per CTA, keys whose bias and score
+    # up to 152 query tiles take the kernel of one tile per item, more that of two (there with an odd
+    # number of tiles, so a pair of one, and many short items per CTA): keys whose bias and score
     # change inside a 32-key chunk or are -inf, logits that grow by far more than 2^8 along the keys
     # (the running maximum is raised, O rescaled), and a logit scale whose maximum is not the products'
     aw, K, V = _case(B, H, Hkv, S, seed=900 + S + H, n_image=S // 4)
